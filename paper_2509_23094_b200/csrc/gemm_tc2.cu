@@ -941,7 +941,8 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
           finish32(e, v, u2 * 16, pre, ahead);
         }
         if (parts > 0) {
-          // the cluster that finishes reading last puts both counters back for the next launch
+          // the cluster that finishes reading last puts both counters back for the next launch (one that gives up does not:
+          // the next step clears them)
           asm volatile("bar.sync 1, 256;" ::: "memory");
           if (etid == 0) {
             int32_t* cnt = g.sk_counters + (g0 * tl.GS + member) * 2 + (int)rank;

@@ -1,5 +1,7 @@
 """The error contract of the C ABI on a device: the status word a kernel's bounded wait writes, what
 d2c_sync_status reports from it, and the argument checks that need a live context."""
+from dataclasses import replace
+
 import pytest
 import torch
 
@@ -60,3 +62,32 @@ def test_a_context_keeps_the_batch_and_length_of_its_first_step():
     assert e.value.code == binding.D2C_EINVAL
     g = pair.gpu_step(wl.k, wl.p)                                   # the original shape still works
     assert len(g["sel"][0]) > 0
+
+
+def test_counts_left_by_a_wait_that_gave_up_do_not_reach_the_next_step():
+    """A projection whose bounded wait ran out leaves the counters of its shared items as they are; a later launch that
+    trusted them would add parts of another launch.  Every step starts with cleared ones: the same bits, whatever is there."""
+    shape, seq = replace(inputs.TOY_HD128, name="deep", d_model=1024, d_ffn=2880, n_q_heads=8, n_kv_heads=8, vocab=4106), 701
+    wl = inputs.Workload("deep", shape, 1, seq, 8, seq - 8, "all", 0, 0.0, seed=5)
+    w = inputs.make_weights(shape, seed=5, device="cuda", gain_jitter=0.05)
+    mask = inputs.make_mask(wl)
+    h0, mask = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask)).cuda(), mask.cuda()
+    conf0 = inputs.make_scores(seq, 7).view(1, seq).cuda()
+    ctx = binding.Context(binding.make_config(shape, 1, seq), w)
+    n = 2 * 320                                                     # arrival and done counters, right before gemm_clocks
+    counters = ctx._view(ctx.state.gemm_clocks - 4 * n, n, torch.int32)
+    hid = torch.zeros(seq, shape.d_model, dtype=torch.bfloat16, device="cuda")
+    ctx.step(h0, mask, seq, 1.0)
+    for rows in (257, 96):                                          # shared between clusters with many and with few rows
+        runs = []
+        for left in (None, 0, 1, 1000):
+            if left is not None:
+                counters.fill_(left)
+            ctx.view("conf", 1, seq).copy_(conf0)
+            hid.zero_()
+            ctx.step(h0, mask, rows, 0.0, hidden_out=hid)
+            ctx.sync_status()
+            assert not counters.any()
+            runs.append([hid.clone(), ctx.view("kcache").clone(), ctx.view("conf").clone(), ctx.view("c").clone()])
+        for other in runs[2:]:                                      # (the first step expects other rows than it finds)
+            assert all(torch.equal(a, b) for a, b in zip(other, runs[1]))
