@@ -92,7 +92,6 @@ struct SelectArgs {
   int32_t* slot_of_pos;
   int32_t* rank_s; int32_t* rank_lm; int32_t* n_b; int32_t* nm_b;   // scratch [B][L],[B][L],[B],[B]
   int32_t* n_host;                               // optional: device-visible address of a host word that receives the total row count
-  int32_t* clear; int n_clear;                   // words set to 0 on the way (null: none)
 };
 int launch_select(const SelectArgs& a, cudaStream_t st);
 // Fills tab[0..len) with floor(exp(-r^2/(2 sigma^2)) * 2^30 + 0.5); returns the first r whose entry is 0 (or len).
@@ -101,7 +100,7 @@ int build_phi_table(float sigma, uint32_t* tab, int len);
 // ---- row kernels (rows.cu) -------------------------------------------------------------------
 int launch_gather_norm(const bf16* h0, const int32_t* sel_idx, const int32_t* row_seq, const int32_t* n_rows,
                        int max_rows, int seq_len, int d, const bf16* gain, float eps, bf16* x, bf16* xn,
-                       cudaStream_t st);
+                       int32_t* clear, int n_clear, cudaStream_t st);       // clear: words set to 0 on the way
 int launch_rmsnorm(const bf16* x, const int32_t* row_map, const int32_t* n_rows, int max_rows, int d,
                    const bf16* gain, float eps, bf16* xn, cudaStream_t st);
 // d2c_step_host's results: rows of x (the live ones) and up to four word arrays, written straight to device-visible host memory

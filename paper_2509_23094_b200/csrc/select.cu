@@ -247,8 +247,6 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
   for (int r = tid; r < min(a.phi_len, kPhiMax); r += kSelThreads) s_phi[r] = a.phi_q30[r];
   for (int i = tid; i < 3 * 256; i += kSelThreads) (&rsc.hist[0][0])[i] = 0;
   if (tid == 0) { s_nm = 0; s_mass = 0; s_lo = 0xFFFFFFFFu; s_hi = 0u; }
-  if (b == 0)
-    for (int i = tid; i < a.n_clear; i += kSelThreads) a.clear[i] = 0;
   __syncthreads();
 
   // ---- the set stage 1 ranks: masked positions inside the block, listed in any order ----
