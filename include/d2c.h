@@ -279,9 +279,10 @@ int d2c_op_rollout(const float* abar, size_t layer_stride, int32_t n_layers, con
 /* The library's bounded device-side wait, on its own.  Every pipeline wait of the tcgen05 kernels (on an
  * mbarrier that a TMA copy or a tensor-core commit completes) gives up after a cycle limit, records
  * D2C_ETIMEOUT in status[0] and the number of the wait that ran out in status[1], and lets the kernel drain
- * and return; d2c_sync_status then reports it.  This entry launches one small CTA that waits, with the given
- * limit (1e3 .. 2e9 SM clocks), on a barrier nothing arrives on: it returns after about that many clocks and
- * leaves status = {D2C_ETIMEOUT, 99, ...}.  status: device int32[4], zeroed by the caller.  It exists so that
+ * and return; d2c_sync_status then reports it.  This entry launches one small CTA in which a warp waits, with the given
+ * limit (1e3 .. 2e9 SM clocks), on a barrier nothing arrives on, while 256 threads meet over and over until they learn
+ * of it: it returns after about that many clocks and leaves status = {D2C_ETIMEOUT, 99, how many of the 256 left
+ * together, ...}.  status: device int32[4], zeroed by the caller.  It exists so that
  * the error path of section "Conventions" can be exercised without a fault; it has no counterpart in the paper. */
 int d2c_op_wait_probe(int32_t* status, int64_t limit_cycles, void* cuda_stream);
 

@@ -268,8 +268,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA128, const __grid_constant
       const bool got = __all_sync(0xffffffffu, mbar_wait(acc_full(buf), use & 1, abortp, status, 3));
       if (S > 1) {
         // ... and, where the four warps meet at named barriers below, for all of them together
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (*abortp) break;
+        if (meet_or_leave<1, 128>(!got)) break;
       } else if (!got) {
         break;
       }
@@ -309,8 +308,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA128, const __grid_constant
             }
           }
         }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (*abortp) break;
+        if (meet_or_leave<1, 128>(*abortp != 0)) break;
         __threadfence();
         reduce = true;
       }

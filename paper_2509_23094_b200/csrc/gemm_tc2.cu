@@ -823,9 +823,8 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
       if (kind != WARM) {
         // a wait that gave up ends the loop for the whole warp (the tcgen05.ld below is warp-collective) and, since the
         // epilogue warps meet at named barriers, for all of them together
-        mbar_wait(acc_full(buf), use & 1, abortp, status, 33);
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (*abortp) break;
+        const bool got = mbar_wait(acc_full(buf), use & 1, abortp, status, 33);
+        if (meet_or_leave<1, 256>(!got)) break;
         tc_fence_after();
         if (kind != FULL) {
           // ---- a part of a split item: park what the other contributors will finish
@@ -887,8 +886,7 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
             }
             __threadfence();
           }
-          asm volatile("bar.sync 1, 256;" ::: "memory");
-          if (*abortp) break;
+          if (meet_or_leave<1, 256>(*abortp != 0)) goto leave;
         }
         const EpiTile e = job();
 #pragma unroll 1
@@ -952,8 +950,8 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
           release_acc();
         }
       }
-      if (*abortp) break;
     }
+  leave:;
   }
   // ------------------------------------------------------------------ teardown
   tc_fence_before();

@@ -54,6 +54,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int site) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, site));
 }
+// Barrier `id` of `threads` threads (whole warps) at which they agree on giving up: true in all of them if one came with
+// `gave_up`.  The abort flag itself does not do for that: another warp may set it between two threads' reads behind a barrier,
+// and who stays then waits for good, at the next barrier, for those that left.  (A vote or a warp barrier before it, or the
+// form for split warps, costs 0.05 us a launch: small steps 0.4 %.)
+template <int id, int threads>
+__device__ __forceinline__ bool meet_or_leave(bool gave_up) {
+  const int mine = gave_up;
+  uint32_t any;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %3, 0;\n\tbarrier.cta.red.or.pred.aligned q, %1, %2, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+               : "=r"(any) : "n"(id), "n"(threads), "r"(mine) : "memory");
+  return any != 0;
+}
 // 1 in one lane of a converged warp.  The warps that issue tcgen05 instructions run their loops with all lanes and
 // predicate only the instruction itself: under a divergent `if (lane == 0)` every descriptor word of every MMA goes
 // through its own move to a uniform register first, which made an MMA cost about 58 clocks of issue.

@@ -47,6 +47,16 @@ def test_a_bounded_wait_that_runs_out_returns_and_records_the_timeout():
         binding.d2c_op_wait_probe(status, limit_cycles=10)          # limits outside [1e3, 2e9] are refused on the host
 
 
+def test_threads_that_meet_leave_together_when_a_wait_gives_up():
+    """Another warp's wait runs out while 256 threads go from one named barrier to the next: whenever the flag is set, all of
+    them leave at the same one (a thread that stayed would wait there for good)."""
+    for limit in (1000, 1234, 5000, 20011, 100003, 1000003):
+        for _ in range(20):
+            status = torch.zeros(4, dtype=torch.int32, device="cuda")
+            binding.d2c_op_wait_probe(status, limit_cycles=limit)
+            assert status.tolist() == [binding.D2C_ETIMEOUT, 99, 256, 0]
+
+
 def test_a_context_keeps_the_batch_and_length_of_its_first_step():
     wl = inputs.WORKLOADS["toy"]
     pair = Pair(wl, max_batch=2, max_seq=wl.seq_len + 64)
