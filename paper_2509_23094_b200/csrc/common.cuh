@@ -58,8 +58,19 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     D2C_CUDA_OK(d2c::launch_pdl(kernel, grid, block, smem, st, __VA_ARGS__));               \
     d2c::count_launch(1);                                                                   \
   } while (0)
-// After a kernel launch: checks the launch and counts it.
-#define D2C_LAUNCHED() do { D2C_CUDA_OK(cudaGetLastError()); d2c::count_launch(1); } while (0)
+// The same without the attribute: the kernel starts when all work before it in the stream is done.  (Either way the launch's own
+// return code is checked; the thread's last error may be an older one, of the caller's.)
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_plain(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
+}
+#define D2C_LAUNCH_PLAIN(kernel, grid, block, smem, st, ...)                                \
+  do {                                                                                      \
+    D2C_CUDA_OK(d2c::launch_plain(kernel, grid, block, smem, st, __VA_ARGS__));             \
+    d2c::count_launch(1);                                                                   \
+  } while (0)
 
 // Per-device one-time set-up (function attributes, device properties): kernels' attributes belong to the
 // device they were set on, so the "done" flags are kept per device ordinal, for the device that is current.

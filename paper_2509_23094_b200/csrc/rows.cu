@@ -90,8 +90,7 @@ rows_to_host_kernel(const uint4* __restrict__ x, const int32_t* __restrict__ n_r
 }
 int launch_rows_to_host(const bf16* x, const int32_t* n_rows, int d, void* dst, cudaStream_t st) {
   // a few warps keep the link busy: 32 CTAs beside whatever runs
-  rows_to_host_kernel<<<32, kRowThreads, 0, st>>>(reinterpret_cast<const uint4*>(x), n_rows, d >> 3, reinterpret_cast<uint4*>(dst));
-  D2C_LAUNCHED();
+  D2C_LAUNCH_PLAIN((rows_to_host_kernel), 32, kRowThreads, 0, st, reinterpret_cast<const uint4*>(x), n_rows, d >> 3, reinterpret_cast<uint4*>(dst));
   return D2C_OK;
 }
 
@@ -125,8 +124,7 @@ __global__ void rope_table_kernel(float2* tab, int max_seq, int half, double bas
 
 int launch_rope_table(float2* tab, int max_seq, int head_dim, float base, cudaStream_t st) {
   const int half = head_dim / 2, n = max_seq * half;
-  rope_table_kernel<<<ceil_div(n, 256), 256, 0, st>>>(tab, max_seq, half, (double)base, head_dim);
-  D2C_LAUNCHED();
+  D2C_LAUNCH_PLAIN((rope_table_kernel), ceil_div(n, 256), 256, 0, st, tab, max_seq, half, (double)base, head_dim);
   return D2C_OK;
 }
 

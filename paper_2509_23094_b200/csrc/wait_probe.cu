@@ -41,7 +41,6 @@ extern "C" int d2c_op_wait_probe(int32_t* status, int64_t limit_cycles, void* cu
     set_global_error("d2c_op_wait_probe: limit_cycles %lld outside [1e3, 2e9]", (long long)limit_cycles);
     return D2C_EINVAL;
   }
-  wait_probe_kernel<<<1, kMeeting + 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(reinterpret_cast<int*>(status), (long long)limit_cycles);
-  D2C_LAUNCHED();
+  D2C_LAUNCH_PLAIN((wait_probe_kernel), 1, kMeeting + 32, 0, static_cast<cudaStream_t>(cuda_stream), reinterpret_cast<int*>(status), (long long)limit_cycles);
   return D2C_OK;
 }

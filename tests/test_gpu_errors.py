@@ -1,5 +1,6 @@
 """The error contract of the C ABI on a device: the status word a kernel's bounded wait writes, what
 d2c_sync_status reports from it, and the argument checks that need a live context."""
+import contextlib
 from dataclasses import replace
 
 import pytest
@@ -101,3 +102,28 @@ def test_counts_left_by_a_wait_that_gave_up_do_not_reach_the_next_step():
             runs.append([hid.clone(), ctx.view("kcache").clone(), ctx.view("conf").clone(), ctx.view("c").clone()])
         for other in runs[2:]:                                      # (the first step expects other rows than it finds)
             assert all(torch.equal(a, b) for a, b in zip(other, runs[1]))
+
+
+def test_an_older_error_of_the_caller_is_not_taken_for_a_launch_error():
+    """The thread's last CUDA error may be the caller's own, of a call that has nothing to do with the library."""
+    def older():                                                    # refused, and remembered as the last error
+        assert int(torch.cuda.cudart().cudaHostUnregister(torch.zeros(8).data_ptr())) != 0
+    shape, seq = inputs.TOY_HD128, 333
+    wl = inputs.Workload("host", shape, 1, seq, 200, 90, "random", 16, 0.2, seed=6)
+    w, status = inputs.make_weights(shape, seed=6, device="cuda"), torch.zeros(4, dtype=torch.int32, device="cuda")
+    mask = inputs.make_mask(wl)
+    h0 = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask))
+    torch.empty(1 << 28, dtype=torch.uint8, device="cuda")          # torch keeps this for the workspace
+    older()
+    ctx = binding.Context(binding.make_config(shape, 1, seq), w)
+    h0, mask = h0.contiguous().pin_memory(), mask.contiguous().pin_memory()
+    hid, off = torch.zeros(seq, shape.d_model, dtype=torch.bfloat16).pin_memory(), torch.zeros(2, dtype=torch.int32).pin_memory()
+    ctx.step_host(h0, mask, seq, 1.0)
+    for _ in range(4):                                              # buffers in place once few rows are expected
+        older()
+        ctx.step_host(h0, mask, 16, 0.1, hidden_out=hid, row_off=off)
+    older()
+    binding.d2c_op_wait_probe(status, limit_cycles=1000)
+    with contextlib.suppress(RuntimeError):                         # (torch reports the older error once and forgets it)
+        torch.zeros(1, device="cuda").add_(1)
+    assert status.tolist()[:2] == [binding.D2C_ETIMEOUT, 99]
