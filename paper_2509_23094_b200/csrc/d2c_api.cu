@@ -700,8 +700,8 @@ int d2c_profile_read(d2c_ctx* ctx, float* phase_ms, int64_t* phase_launches, int
 
 const char* d2c_phase_name(int32_t i) { return (i >= 0 && i < D2C_N_PHASES) ? kPhaseNames[i] : ""; }
 
-int d2c_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_host_out* out) {
-  D2C_TRY(ctx, check_step_args(ctx, h));
+// Enqueues the copies and the step of a host call.
+static int enqueue_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_host_out* out) {
   const d2c_config& c = ctx->cfg;
   const Buffers& b = ctx->buf;
   cudaStream_t st = ctx->stream;
@@ -735,8 +735,7 @@ int d2c_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_host_out* out)
        if (!a.field) return fail(ctx, D2C_ECUDA, "d2c_step_host: copying %s failed: %s", #field, cudaGetErrorString(cudaGetLastError())); } while (0)
   D2C_IN(mask, b.mask_stage, R);
   if (h->forced) {
-    int32_t n_forced = h->forced_off[B];
-    if (n_forced < 0 || (size_t)n_forced > R) return fail(ctx, D2C_EINVAL, "d2c_step_host: %d forced rows", n_forced);
+    const int32_t n_forced = h->forced_off[B];
     D2C_IN(forced_off, b.forced_off_stage, (B + 1) * sizeof(int32_t));
     if (n_forced) D2C_IN(forced, b.forced_stage, (size_t)n_forced * sizeof(int32_t));
     else a.forced = b.forced_stage;
@@ -751,7 +750,7 @@ int d2c_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_host_out* out)
   if (reinterpret_cast<uintptr_t>(ctx->early_hidden_dev) % 16) ctx->early_hidden_dev = nullptr;
   const int step_rc = d2c_step(ctx, &a, &dev_out);
   ctx->early_hidden_host = ctx->early_hidden_dev = nullptr;
-  if (step_rc != D2C_OK) { if (early) cudaStreamSynchronize(ctx->copy_stream); return step_rc; }
+  if (step_rc != D2C_OK) return step_rc;
   // every other result is copied without knowing the row count (worst-case sizes), then one synchronisation
   if (out) {
     const void* src[4] = {b.row_off, b.sel_idx, b.conf, b.pred};
@@ -770,11 +769,23 @@ int d2c_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_host_out* out)
     if (any) D2C_TRY(ctx, launch_results_to_host(hr, st));
     if (out->hidden_out_host && !early) D2C_CP(out->hidden_out_host, b.x, R * c.d_model * sizeof(bf16), cudaMemcpyDeviceToHost);
   }
-  cudaError_t e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && early) e = cudaStreamSynchronize(ctx->copy_stream);
-  if (e != cudaSuccess) return fail(ctx, D2C_ECUDA, "d2c_step_host: %s", cudaGetErrorString(e));
 #undef D2C_CP
   return D2C_OK;
+}
+
+int d2c_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_host_out* out) {
+  D2C_TRY(ctx, check_step_args(ctx, h));
+  if (h->forced && (h->forced_off[h->batch] < 0 || (size_t)h->forced_off[h->batch] > (size_t)h->batch * h->seq_len))
+    return fail(ctx, D2C_EINVAL, "d2c_step_host: %d forced rows", h->forced_off[h->batch]);
+  const int rc = enqueue_step_host(ctx, h, out);
+  // The caller may free its buffers once it has the answer, also when that is an error: nothing enqueued so far may use them
+  // any longer.  (Behind an error the step's own streams need not have been joined.)
+  cudaError_t e = cudaStreamSynchronize(ctx->stream);
+  if (ctx->copy_stream && out && out->hidden_out_host) { const cudaError_t e2 = cudaStreamSynchronize(ctx->copy_stream); if (e == cudaSuccess) e = e2; }
+  if (rc == D2C_OK) return e == cudaSuccess ? D2C_OK : fail(ctx, D2C_ECUDA, "d2c_step_host: %s", cudaGetErrorString(e));
+  if (ctx->work_stream) { cudaStreamSynchronize(ctx->work_stream); cudaStreamSynchronize(ctx->side_stream); }
+  (void)cudaGetLastError();                                  // reported by this call, not to whoever asks next
+  return rc;
 }
 
 int d2c_commit(d2c_ctx* ctx, int32_t batch, int32_t seq_len, const void* embed_table, void* h0,

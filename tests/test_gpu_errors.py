@@ -1,6 +1,8 @@
 """The error contract of the C ABI on a device: the status word a kernel's bounded wait writes, what
 d2c_sync_status reports from it, and the argument checks that need a live context."""
 import contextlib
+import ctypes
+import mmap
 from dataclasses import replace
 
 import pytest
@@ -127,3 +129,40 @@ def test_an_older_error_of_the_caller_is_not_taken_for_a_launch_error():
     with contextlib.suppress(RuntimeError):                         # (torch reports the older error once and forgets it)
         torch.zeros(1, device="cuda").add_(1)
     assert status.tolist()[:2] == [binding.D2C_ETIMEOUT, 99]
+
+
+def test_a_host_call_that_fails_late_has_let_go_of_its_buffers():
+    """The copy of the last result is refused (its buffer is registered in part) when the step is already enqueued: when the
+    call comes back with its error, nothing that it enqueued runs any more, and the error is not left for the next caller."""
+    shape, batch, seq = inputs.TOY, 3, 8192                          # (results above 64 KB are copied)
+    wl = inputs.Workload("late", shape, batch, seq, 8000, 100, "random", 16, 0.1, seed=6)
+    w = inputs.make_weights(shape, seed=6, device="cuda")
+    mask = inputs.make_mask(wl)
+    h0 = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask)).contiguous().pin_memory()
+    mask, hid = mask.contiguous().pin_memory(), torch.zeros(batch * seq, shape.d_model, dtype=torch.bfloat16).pin_memory()
+    off = torch.zeros(batch + 1, dtype=torch.int32).pin_memory()
+    conf = torch.zeros(batch, seq).pin_memory()
+    ctx = binding.Context(binding.make_config(shape, batch, seq), w)
+    ctx.step_host(h0, mask, seq, 1.0, hidden_out=hid, row_off=off, conf=conf)
+    want = hid.clone()
+    mem = mmap.mmap(-1, batch * seq * 4)
+    base, rt = ctypes.addressof(ctypes.c_char.from_buffer(mem)), torch.cuda.cudart()
+    assert int(rt.cudaHostRegister(base, mmap.PAGESIZE, 0)) == 0
+    try:
+        part = torch.frombuffer(mem, dtype=torch.float32).view(batch, seq)
+        hid.zero_()
+        with pytest.raises(binding.D2cError) as e:
+            ctx.step_host(h0, mask, seq, 1.0, hidden_out=hid, row_off=off, conf=part)
+        idle = torch.cuda.current_stream().query()
+        assert e.value.code == binding.D2C_ECUDA and idle
+        assert torch.equal(hid, want)                                # it had been copied, and will not change any more
+        assert int(torch.zeros(4, device="cuda").add_(1).sum()) == 4
+        with pytest.raises(binding.D2cError) as e:                   # a bad count is refused before anything is enqueued
+            ctx.step_host(h0, mask, 4, 0.1, forced=torch.zeros(1, dtype=torch.int32), forced_off=torch.tensor([0, 0, 0, -1], dtype=torch.int32))
+        assert e.value.code == binding.D2C_EINVAL and torch.cuda.current_stream().query()
+        hid.zero_()
+        ctx.step_host(h0, mask, seq, 1.0, hidden_out=hid, row_off=off, conf=conf)
+        assert torch.equal(hid, want)
+    finally:
+        torch.cuda.synchronize()
+        rt.cudaHostUnregister(base)
