@@ -1,5 +1,6 @@
 // C-ABI layer of the d2Cache step: argument validation, the carve-up of the caller's workspace and
 // the launch sequence of one step.  No device memory is allocated here.
+#include <cuda.h>
 #include <math.h>
 #include <stdarg.h>
 #include <string.h>
@@ -224,6 +225,30 @@ static int cu(cudaError_t e) {
   if (e == cudaSuccess) return D2C_OK;
   set_global_error("d2c_step: %s", cudaGetErrorString(e));
   return D2C_ECUDA;
+}
+// The device's address of a host buffer that kernels may use in place: all of its bytes lie in one pinned allocation or
+// registration (the first byte's attributes are not enough: a registered range may end inside the buffer, and a kernel that
+// runs past it faults where a copy returns an error), and it starts at a word.  Null for every other buffer, which is copied.
+static void* mapped(const void* p, size_t bytes) {
+  typedef CUresult (*GetAttributes)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+  static GetAttributes get = []() -> GetAttributes {                       // (the library does not link libcuda)
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
+    if (!ok) (void)cudaGetLastError();
+    return ok ? reinterpret_cast<GetAttributes>(fn) : nullptr;
+  }();
+  cudaPointerAttributes at;
+  if (!p || bytes == 0 || !get) return nullptr;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { (void)cudaGetLastError(); return nullptr; }
+  if (at.type != cudaMemoryTypeHost || !at.devicePointer || reinterpret_cast<uintptr_t>(at.devicePointer) % 4) return nullptr;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[2] = {&start, &size};
+  const CUdeviceptr first = reinterpret_cast<CUdeviceptr>(at.devicePointer);
+  if (get(2, what, to, first) != CUDA_SUCCESS) return nullptr;
+  return first >= start && first - start <= size && bytes <= size - (first - start) ? at.devicePointer : nullptr;
 }
 #define D2C_TRY(ctx, expr) do { int rc__ = (expr); if (rc__ != D2C_OK) return pass((ctx), rc__); } while (0)
 
@@ -713,20 +738,14 @@ static int enqueue_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_hos
   // the link, the gather only the selected rows of h0 and the copy at the end only those rows.  A copy engine moves whole
   // arrays faster, so h0 and the hidden rows go that way when most rows are expected (one layer, 1024 rows of 8 KB, 116
   // selected: 150 us of copies saved on each side; a transfer of all rows by kernels is no faster than the engine's).
-  auto mapped = [](const void* p) -> void* {
-    cudaPointerAttributes at;
-    if (p && cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeHost) return at.devicePointer;
-    (void)cudaGetLastError();
-    return nullptr;
-  };
   d2c_step_args a = *h;
   const size_t few = R / 2;
   const bool few_expected = (size_t)ctx->last_rows <= few;
-  const void* h0_dev = few_expected ? mapped(h->h0) : nullptr;
+  const void* h0_dev = few_expected ? mapped(h->h0, R * c.d_model * sizeof(bf16)) : nullptr;
   if (h0_dev && reinterpret_cast<uintptr_t>(h0_dev) % 16 == 0) a.h0 = h0_dev;
   else { D2C_CP(b.h0_stage, h->h0, R * c.d_model * sizeof(bf16), cudaMemcpyHostToDevice); a.h0 = b.h0_stage; }
   auto input = [&](const void* src, void* stage, size_t bytes) -> const void* {
-    if (const void* p = bytes <= 64 * 1024 ? mapped(src) : nullptr) return p;
+    if (const void* p = bytes <= 64 * 1024 ? mapped(src, bytes) : nullptr) return p;
     const cudaError_t e = cudaMemcpyAsync(stage, src, bytes, cudaMemcpyHostToDevice, st);
     return e == cudaSuccess ? stage : nullptr;
   };
@@ -746,7 +765,7 @@ static int enqueue_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_hos
   d2c_step_out dev_out{};
   const bool early = out && out->hidden_out_host && ctx->copy_stream;
   ctx->early_hidden_host = early ? out->hidden_out_host : nullptr;
-  ctx->early_hidden_dev = early && few_expected ? mapped(out->hidden_out_host) : nullptr;
+  ctx->early_hidden_dev = early && few_expected ? mapped(out->hidden_out_host, R * c.d_model * sizeof(bf16)) : nullptr;
   if (reinterpret_cast<uintptr_t>(ctx->early_hidden_dev) % 16) ctx->early_hidden_dev = nullptr;
   const int step_rc = d2c_step(ctx, &a, &dev_out);
   ctx->early_hidden_host = ctx->early_hidden_dev = nullptr;
@@ -760,7 +779,7 @@ static int enqueue_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_hos
     bool any = false;
     for (int k = 0; k < 4; ++k) {
       if (!dst[k]) continue;
-      if (void* p = n[k] * 4 <= 64 * 1024 ? mapped(dst[k]) : nullptr) {
+      if (void* p = n[k] * 4 <= 64 * 1024 ? mapped(dst[k], n[k] * 4) : nullptr) {
         hr.src[k] = static_cast<const uint32_t*>(src[k]); hr.dst[k] = static_cast<uint32_t*>(p); hr.n[k] = (int)n[k]; any = true;
       } else {
         D2C_CP(dst[k], src[k], n[k] * 4, cudaMemcpyDeviceToHost);

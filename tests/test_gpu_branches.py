@@ -202,3 +202,87 @@ def test_top_p_crossing_bin(m, step, ties, far):
         want, _, _ = oselection.select_rows(mask, np.full(L, 0.5, np.float32), c, 4, p, 10.0)
         n = int(out["row_off"][1])
         np.testing.assert_array_equal(out["sel_idx"][:n].cpu().numpy(), want, err_msg=str((frac, p)))
+
+
+@pytest.mark.parametrize("name", ["h0", "mask", "scores", "hidden", "conf", "pred"])
+@pytest.mark.parametrize("split", [False, True])
+def test_host_buffers_registered_in_part(name, split):
+    """A buffer of which only the first page is registered, or whose registration comes in two pieces, is not used in place:
+    the copy says so with an error code, as it does for any such buffer, and the context goes on."""
+    import ctypes
+    import mmap
+    shape, seq = inputs.TOY_HD128, 6000                                # every buffer is longer than a page
+    wl = inputs.Workload("host", shape, 1, seq, 5000, 500, "random", 16, 0.01, seed=6)
+    w = inputs.make_weights(shape, seed=6, device="cuda", gain_jitter=0.05)
+    mask = inputs.make_mask(wl)
+    h0 = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask))
+    ctx = binding.Context(binding.make_config(shape, 1, seq), w)
+    ctx.step(h0.cuda(), mask.cuda(), seq, 1.0)
+    good = {"h0": h0.contiguous(), "mask": mask.contiguous(), "scores": inputs.make_scores(seq, 8).view(1, seq), "sel": torch.zeros(seq, dtype=torch.int32),
+            "off": torch.zeros(2, dtype=torch.int32), "hidden": torch.zeros(seq, shape.d_model, dtype=torch.bfloat16),
+            "conf": torch.zeros(1, seq), "pred": torch.zeros(1, seq, dtype=torch.int32)}
+    good = {k: v.pin_memory() for k, v in good.items()}
+
+    def call(t):
+        ctx.step_host(t["h0"], t["mask"], 16, 0.01, override_c=t["scores"], sel_idx=t["sel"], row_off=t["off"], hidden_out=t["hidden"],
+                      conf=t["conf"], pred=t["pred"])
+        n = int(t["off"][1])
+        return [x.clone() for x in (t["sel"][:n], t["off"], t["hidden"][:n], t["conf"], t["pred"])]
+    for _ in range(3):                                                 # few rows expected: the pinned buffers serve in place
+        want = call(good)
+    nbytes = good[name].numel() * good[name].element_size()
+    page, rt = mmap.PAGESIZE, torch.cuda.cudart()
+    pages = -(-nbytes // page)
+    assert pages > 1
+    mem = mmap.mmap(-1, pages * page)
+    base = ctypes.addressof(ctypes.c_char.from_buffer(mem))
+    pieces = [(base, page)] + ([(base + page, (pages - 1) * page)] if split else [])
+    for at, size in pieces:
+        assert int(rt.cudaHostRegister(at, size, 0)) == 0
+    try:
+        part = torch.frombuffer(mem, dtype=good[name].dtype, count=good[name].numel()).view(good[name].shape)
+        part.copy_(good[name])
+        try:
+            got = call({**good, name: part})                           # (a driver that takes such a copy gives the results)
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+        except binding.D2cError as e:
+            assert e.code == binding.D2C_ECUDA
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(call(good), want))
+    finally:
+        torch.cuda.synchronize()
+        for at, _ in pieces:
+            rt.cudaHostUnregister(at)
+
+
+def test_host_buffers_off_their_alignment():
+    """Pinned buffers that do not start at a word (or at 16 bytes, for the rows) are copied: the same results."""
+    shape, seq = inputs.TOY_HD128, 333
+    wl = inputs.Workload("host", shape, 1, seq, 200, 90, "random", 16, 0.2, seed=6)
+    w = inputs.make_weights(shape, seed=6, device="cuda", gain_jitter=0.05)
+    mask = inputs.make_mask(wl)
+    h0 = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask))
+    data = [h0, mask, inputs.make_scores(seq, 8).view(1, seq), torch.tensor([3], dtype=torch.int32), torch.tensor([0, 1], dtype=torch.int32)]
+    sizes = [4 * seq, 8, 2 * seq * shape.d_model, 4 * seq, 4 * seq]                 # sel_idx, row_off, hidden, conf, pred
+    results = []
+    for shift in (0, 2, 1):
+        ctx = binding.Context(binding.make_config(shape, 1, seq), w)
+        ctx.step(h0.cuda(), mask.cuda(), seq, 1.0)
+        raw = [t.contiguous().view(-1).view(torch.uint8) for t in data]
+        ins = [torch.zeros(t.numel() + 16, dtype=torch.uint8).pin_memory() for t in raw]
+        for t, r in zip(ins, raw):
+            t[shift: shift + r.numel()] = r
+        outs = [torch.zeros(n + 16, dtype=torch.uint8).pin_memory() for n in sizes]
+        at = [t.data_ptr() + (shift if i != 4 else 0) for i, t in enumerate(ins)]   # (the host reads forced_off itself)
+        if shift:
+            ins[4][: raw[4].numel()] = raw[4]
+        to = [t.data_ptr() + shift for t in outs]
+        a = binding.StepArgs(1, seq, at[0], at[1], at[3], at[4], 16, 0.2, None, at[2], 0, 0)
+        for _ in range(4):
+            binding._check(binding.load().d2c_step_host(ctx.handle, a, binding.HostOut(to[0], to[1], to[2], to[3], to[4])), ctx.handle)
+        got = [t[shift: shift + n].clone() for t, n in zip(outs, sizes)]
+        n = int(got[1].view(torch.int32)[1])
+        results.append([got[0][: 4 * n], got[1], got[2][: 2 * n * shape.d_model], got[3], got[4]])
+        assert 0 < n < seq // 2
+    for other in results[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(other, results[0]))
