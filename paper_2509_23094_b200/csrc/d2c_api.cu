@@ -147,7 +147,6 @@ struct d2c_ctx {
   cudaEvent_t layers_done = nullptr;
   void* early_hidden_host = nullptr;     // set by d2c_step_host for the duration of one step
   void* early_hidden_dev = nullptr;      // the same buffer as the device sees it: only the live rows are written (null: copy all)
-  int last_rows = 1 << 30;               // the row count a step last went by (see expect_rows)
   // The head-averaged probabilities and the rollout feed only the next step's selection.  They run on a
   // low-priority stream beside the projections, the FFN and the LM head, filling the SMs those leave idle
   // (partial last waves); the rest of the step runs on a high-priority stream so that it wins every SM it
@@ -386,6 +385,20 @@ static int check_step_args(d2c_ctx* ctx, const d2c_step_args* a) {
   return D2C_OK;
 }
 
+static bool stream_captures(const d2c_ctx* ctx) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess) { (void)cudaGetLastError(); return true; }
+  return cs != cudaStreamCaptureStatusNone;
+}
+// The row count of the step before, read behind that step's selection kernel, which the next one goes by; left alone if there is none.
+static int previous_rows(d2c_ctx* ctx, bool capturing, int* rows) {
+  const int prev = (int)(ctx->step_no & 1) ^ 1;
+  if (!ctx->hint_host[0] || capturing || ctx->hint_step[prev] != ctx->step_no - 1) return D2C_OK;
+  const int rc = cu(cudaEventSynchronize(ctx->ev_hint[prev]));
+  if (rc == D2C_OK) *rows = *reinterpret_cast<volatile int32_t*>(ctx->hint_host[prev]);
+  return rc;
+}
+
 int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   D2C_TRY(ctx, check_step_args(ctx, a));
   const d2c_config& c = ctx->cfg;
@@ -404,21 +417,11 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   // leave alone.  Otherwise a statically scheduled GEMM whose CTAs start late behind side-stream CTAs loses more than the
   // overlap gains (measured at 488 rows x 32 layers: +5 %).
   // regime of this step: the row count of the previous step, read behind that step's selection kernel
-  bool capturing = false;
-  {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess) { (void)cudaGetLastError(); capturing = true; }
-    else capturing = cs != cudaStreamCaptureStatusNone;
-  }
-  const bool track = ctx->hint_host[0] != nullptr && !capturing;
-  const int slot = (int)(ctx->step_no & 1), prev = slot ^ 1;
+  const bool capturing = stream_captures(ctx), track = ctx->hint_host[0] != nullptr && !capturing;
+  const int slot = (int)(ctx->step_no & 1);
   int expect_rows = 1 << 30;
-  if (track && ctx->hint_step[prev] == ctx->step_no - 1) {
-    D2C_TRY(ctx, cu(cudaEventSynchronize(ctx->ev_hint[prev])));
-    expect_rows = *reinterpret_cast<volatile int32_t*>(ctx->hint_host[prev]);
-  }
+  D2C_TRY(ctx, previous_rows(ctx, capturing, &expect_rows));
   ctx->few_rows = expect_rows <= 128;
-  ctx->last_rows = expect_rows;
   const bool few_rows = ctx->few_rows;
   // With few rows the projections stream weights and 96 of the 148 SMs take all the HBM gives (32 layers at 81 rows: 64
   // pairs 4.60 ms, 48 pairs 4.77), while a projection whose share of SMs is held by the probabilities pass waits for it
@@ -736,11 +739,13 @@ static int enqueue_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_hos
        if (e__ != cudaSuccess) return fail(ctx, D2C_ECUDA, "d2c_step_host: %s", cudaGetErrorString(e__)); } while (0)
   // Pinned buffers are read and written in place by the step's kernels: the selection reads the masks and scores over
   // the link, the gather only the selected rows of h0 and the copy at the end only those rows.  A copy engine moves whole
-  // arrays faster, so h0 and the hidden rows go that way when most rows are expected (one layer, 1024 rows of 8 KB, 116
-  // selected: 150 us of copies saved on each side; a transfer of all rows by kernels is no faster than the engine's).
+  // arrays faster, so h0 and the hidden rows go that way when most rows are expected, going by the step before as d2c_step
+  // does (one layer, 1024 rows of 8 KB, 116 selected: 150 us of copies saved on each side; a transfer of all rows by kernels
+  // is no faster than the engine's).
   d2c_step_args a = *h;
-  const size_t few = R / 2;
-  const bool few_expected = (size_t)ctx->last_rows <= few;
+  int expect_rows = 1 << 30;
+  D2C_TRY(ctx, previous_rows(ctx, stream_captures(ctx), &expect_rows));
+  const bool few_expected = (size_t)expect_rows <= R / 2;
   const void* h0_dev = few_expected ? mapped(h->h0, R * c.d_model * sizeof(bf16)) : nullptr;
   if (h0_dev && reinterpret_cast<uintptr_t>(h0_dev) % 16 == 0) a.h0 = h0_dev;
   else { D2C_CP(b.h0_stage, h->h0, R * c.d_model * sizeof(bf16), cudaMemcpyHostToDevice); a.h0 = b.h0_stage; }

@@ -146,7 +146,7 @@ def test_host_step_in_place():
         o = [pin(t) for t in (torch.full((seq,), -1, dtype=torch.int32), torch.zeros(2, dtype=torch.int32),
                               torch.zeros(seq, shape.d_model, dtype=torch.bfloat16), torch.zeros(1, seq), torch.zeros(1, seq, dtype=torch.int32))]
         got = []
-        for k in (16, 16, 1, 16, 90):                                  # few rows expected from the second on; none before the first
+        for k in (16, 16, 1, 16, 90):                                  # few rows expected from the second on
             ctx.step_host(a[0], a[1], k, 0.2, override_c=a[2], sel_idx=o[0], row_off=o[1], hidden_out=o[2], conf=o[3], pred=o[4])
             n = int(o[1][1])
             got.append([t.clone() for t in (o[0][:n], o[1], o[2][:n], o[3], o[4])])
@@ -202,6 +202,36 @@ def test_top_p_crossing_bin(m, step, ties, far):
         want, _, _ = oselection.select_rows(mask, np.full(L, 0.5, np.float32), c, 4, p, 10.0)
         n = int(out["row_off"][1])
         np.testing.assert_array_equal(out["sel_idx"][:n].cpu().numpy(), want, err_msg=str((frac, p)))
+
+
+def test_host_step_goes_by_the_step_before():
+    """From most rows to few and back: the buffers are used in place by the call behind a step with few rows (only the live
+    rows of the hidden buffer are then written) and copied whole by the one behind a step with most; the same results."""
+    shape, seq = inputs.TOY_HD128, 333
+    wl = inputs.Workload("host", shape, 1, seq, 200, 90, "random", 16, 0.2, seed=6)
+    w = inputs.make_weights(shape, seed=6, device="cuda", gain_jitter=0.05)
+    mask = inputs.make_mask(wl)
+    h0 = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask))
+    scores, results, in_place = inputs.make_scores(seq, 8).view(1, seq), [], []
+    for pin in (lambda t: t.clone().pin_memory(), lambda t: t.clone()):
+        ctx = binding.Context(binding.make_config(shape, 1, seq), w)
+        ctx.step(h0.cuda(), mask.cuda(), seq, 1.0)
+        a = [pin(t) for t in (h0, mask, scores)]
+        o = [pin(t) for t in (torch.zeros(seq, dtype=torch.int32), torch.zeros(2, dtype=torch.int32),
+                              torch.zeros(seq, shape.d_model, dtype=torch.bfloat16), torch.zeros(1, seq), torch.zeros(1, seq, dtype=torch.int32))]
+        got, live = [], []
+        for k, p in ((16, 0.2), (16, 0.2), (90, 0.99), (16, 0.2), (1, 0.01), (1, 0.01)):
+            o[2].fill_(-7.0)
+            ctx.step_host(a[0], a[1], k, p, override_c=a[2], sel_idx=o[0], row_off=o[1], hidden_out=o[2], conf=o[3], pred=o[4])
+            n = int(o[1][1])
+            got.append([t.clone() for t in (o[0][:n], o[1], o[2][:n], o[3], o[4])])
+            live.append(bool((o[2][n:] == -7.0).all()))
+        results.append(got)
+        in_place.append(live)
+    for x, y in zip(*results):
+        for s, t in zip(x, y):
+            assert torch.equal(s, t)
+    assert in_place == [[False, True, True, False, True, True], [False] * 6]
 
 
 @pytest.mark.parametrize("name", ["h0", "mask", "scores", "hidden", "conf", "pred"])
