@@ -404,7 +404,8 @@ __device__ __forceinline__ void finish(const EpiTile& e, float (&v)[32], int tk0
     __syncwarp();
   } else if constexpr (EPI == EPI_LMSTATS) {
     // Per token over the CTA's 128 features: maximum, its lowest index, sum of exp(x - max).  First over this warp's 32
-    // lanes, then over the four warps through their buffers.
+    // lanes, then over the four warps through their buffers.  Features past the end count as -inf, which adds nothing; a
+    // logit that is not a number is no maximum but makes the sum, and with it the confidence, not a number.
     float mx[8], sum[8];
     int arg[8];
 #pragma unroll
@@ -435,8 +436,8 @@ __device__ __forceinline__ void finish(const EpiTile& e, float (&v)[32], int tk0
 #pragma unroll
       for (int r = 3; r >= 0; --r) {                          // (the lowest feature wins)
         const float x = v[i0 + 16 * (r >> 1) + 2 * (r & 1)];
-        if (x == mx[t]) arg[t] = e.f + 8 * r + fr;
-        sum[t] += x > -INFINITY ? __expf(x - mx[t]) : 0.f;
+        if (x == mx[t] && e.f + 8 * r + fr < g.N) arg[t] = e.f + 8 * r + fr;
+        sum[t] += x == -INFINITY ? 0.f : __expf(x - mx[t]);
       }
     }
     int item = 0;                                              // each step also halves the tokens a lane carries
@@ -469,7 +470,7 @@ __device__ __forceinline__ void finish(const EpiTile& e, float (&v)[32], int tk0
       for (int q = 0; q < 4; ++q) {
         const float pm = __uint_as_float(p[q].x);
         if (pm == m) am = min(am, (int)p[q].z);
-        if (pm > -INFINITY) s += __uint_as_float(p[q].y) * __expf(pm - m);
+        s = fmaf(__uint_as_float(p[q].y), pm == -INFINITY ? 1.f : __expf(pm - m), s);
       }
       if (row < e.n && e.stile < g.n_tiles) {
         const size_t o = (size_t)row * g.n_tiles + e.stile;

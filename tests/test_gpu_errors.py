@@ -131,6 +131,34 @@ def test_an_older_error_of_the_caller_is_not_taken_for_a_launch_error():
     assert status.tolist()[:2] == [binding.D2C_ETIMEOUT, 99]
 
 
+@pytest.mark.parametrize("flags", [0, 1, 4])
+def test_logits_that_are_not_numbers_reach_the_confidences(flags):
+    """One row of the LM head that is not a number: every confidence is not a number, and the tokens are the best of the
+    others.  A hidden state that is not a number: no logit has a maximum, and no token is made up from the padding."""
+    shape, seq = replace(inputs.TOY_HD128, vocab=1002), 200          # the last 128 features are not all there
+    wl = inputs.Workload("nan", shape, 1, seq, 100, 60, "random", 16, 0.2, seed=6)
+    w = inputs.make_weights(shape, seed=6, device="cuda")
+    mask = inputs.make_mask(wl)
+    h0, mask = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask)).cuda(), mask.cuda()
+    at = mask[0].nonzero().flatten()
+    def run(w, h0):
+        ctx = binding.Context(binding.make_config(shape, 1, seq, flags=flags), w)
+        ctx.step(h0, mask, seq, 1.0)
+        ctx.sync_status()
+        return ctx.view("conf", 1, seq)[0][at].clone(), ctx.view("pred", 1, seq)[0][at].clone()
+    conf, pred = run(w, h0)
+    assert bool(torch.isfinite(conf).all())
+    bad = dict(w, w_lm=w["w_lm"].clone())
+    unused = next(t for t in range(200, 300) if not bool((pred == t).any()))
+    bad["w_lm"][unused] = float("nan")
+    conf2, pred2 = run(bad, h0)
+    assert bool(torch.isnan(conf2).all()) and torch.equal(pred, pred2)
+    nan_h0 = h0.clone()
+    nan_h0[:] = float("nan")
+    conf3, pred3 = run(w, nan_h0)
+    assert bool(torch.isnan(conf3).all()) and bool((pred3 == 0x7fffffff).all())
+
+
 def test_a_host_call_that_fails_late_has_let_go_of_its_buffers():
     """The copy of the last result is refused (its buffer is registered in part) when the step is already enqueued: when the
     call comes back with its error, nothing that it enqueued runs any more, and the error is not left for the next caller."""
