@@ -159,7 +159,7 @@ int d2c_step_host(d2c_ctx* ctx, const d2c_step_args* host_args, const d2c_host_o
  * score - rule 0: confidence s^i; rule 1: certainty prior D(i)*s^i (Section 4.1).
  * Writes the predicted token into tokens[b][pos], clears mask[b][pos], copies
  * embed_table[token] into h0[b][pos] and records pos in committed[b] (-1 if the
- * sequence has nothing left).  rule 2 commits every such position whose
+ * sequence has nothing left; a row whose logits are not numbers predicts no token and is passed over).  rule 2 commits every such position whose
  * confidence exceeds `threshold` (parallel decoding), at least one per sequence;
  * committed then receives only the best one. */
 int d2c_commit(d2c_ctx* ctx, int32_t batch, int32_t seq_len, const void* embed_table, void* h0,

@@ -1,12 +1,12 @@
 // Decoding-loop helper (Eq. 2): replaces masked positions by their predicted tokens.
 // One CTA per sequence.  Eligible positions are those whose prediction the last step refreshed
-// (selected and still masked).  Scores: confidence s^i, or the certainty prior D(i)*s^i of Section 4.1.
+// (selected and still masked) and is a token: a row whose logits are not numbers predicts none.  Scores: confidence s^i, or the certainty prior D(i)*s^i of Section 4.1.
 #include "common.cuh"
 
 namespace d2c {
 
 struct CommitArgs {
-  int seq_len, d, rule; float threshold;
+  int seq_len, d, vocab, rule; float threshold;
   const int32_t* slot_of_pos; const float* conf; const int32_t* pred; const uint32_t* phi_q30; int phi_len;
   const bf16* embed; bf16* h0; uint8_t* mask; int32_t* tokens; int32_t* committed;
 };
@@ -21,6 +21,7 @@ __global__ void __launch_bounds__(256) commit_kernel(CommitArgs a) {
   for (int j = tid; j < L; j += 256) {
     take[j] = 0;
     if (!mask[j] || a.slot_of_pos[(size_t)b * L + j] < 0) continue;
+    if ((uint32_t)a.pred[(size_t)b * L + j] >= (uint32_t)a.vocab) continue;
     const float s = a.conf[(size_t)b * L + j];
     float score = s;
     if (a.rule == 1) {
@@ -61,10 +62,10 @@ __global__ void __launch_bounds__(256) commit_kernel(CommitArgs a) {
   }
 }
 
-int launch_commit(int batch, int seq_len, int d, int rule, float threshold, const int32_t* slot_of_pos,
+int launch_commit(int batch, int seq_len, int d, int vocab, int rule, float threshold, const int32_t* slot_of_pos,
                   const float* conf, const int32_t* pred, const uint32_t* phi, int phi_len, const bf16* embed,
                   bf16* h0, uint8_t* mask, int32_t* tokens, int32_t* committed, cudaStream_t st) {
-  CommitArgs a{seq_len, d, rule, threshold, slot_of_pos, conf, pred, phi, phi_len, embed, h0, mask, tokens, committed};
+  CommitArgs a{seq_len, d, vocab, rule, threshold, slot_of_pos, conf, pred, phi, phi_len, embed, h0, mask, tokens, committed};
   D2C_LAUNCH((commit_kernel), batch, 256, seq_len, st, a);
   return D2C_OK;
 }

@@ -219,7 +219,7 @@ static const int kRolloutCluster = 8;          // CTAs (SMs) per sequence of the
 
 namespace d2c {
 // ---- commit helper (commit.cu) -------------------------------------------------------------------
-int launch_commit(int batch, int seq_len, int d, int rule, float threshold, const int32_t* slot_of_pos,
+int launch_commit(int batch, int seq_len, int d, int vocab, int rule, float threshold, const int32_t* slot_of_pos,
                   const float* conf, const int32_t* pred, const uint32_t* phi, int phi_len, const bf16* embed,
                   bf16* h0, uint8_t* mask, int32_t* tokens, int32_t* committed, cudaStream_t st);
 // ---- tcgen05 GEMM (gemm_tc.cu) -------------------------------------------------------------------

@@ -822,7 +822,7 @@ int d2c_commit(d2c_ctx* ctx, int32_t batch, int32_t seq_len, const void* embed_t
   if (ctx->used_batch != 0 && (batch != ctx->used_batch || seq_len != ctx->used_seq))
     return fail(ctx, D2C_EINVAL, "d2c_commit: batch %d x seq_len %d differs from the %d x %d of this context's steps", batch, seq_len, ctx->used_batch, ctx->used_seq);
   const Buffers& b = ctx->buf;
-  D2C_TRY(ctx, launch_commit(batch, seq_len, ctx->cfg.d_model, rule, threshold, b.slot_of_pos, b.conf, b.pred, b.phi,
+  D2C_TRY(ctx, launch_commit(batch, seq_len, ctx->cfg.d_model, ctx->cfg.vocab, rule, threshold, b.slot_of_pos, b.conf, b.pred, b.phi,
                              ctx->phi_len < seq_len ? ctx->phi_len : seq_len, (const bf16*)embed_table, (bf16*)h0, mask,
                              tokens, committed, ctx->stream));
   return D2C_OK;

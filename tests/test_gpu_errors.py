@@ -159,6 +159,33 @@ def test_logits_that_are_not_numbers_reach_the_confidences(flags):
     assert bool(torch.isnan(conf3).all()) and bool((pred3 == 0x7fffffff).all())
 
 
+@pytest.mark.parametrize("rule", [0, 1, 2])
+def test_commit_passes_over_rows_that_predict_no_token(rule):
+    """One sequence of two has hidden states that are not numbers: nothing of it is committed (its predictions are no rows of
+    the embedding table), the other goes on as alone."""
+    shape, seq = inputs.TOY_HD128, 200
+    wl = inputs.Workload("nan", shape, 2, seq, 100, 60, "random", 16, 0.2, seed=6)
+    w = inputs.make_weights(shape, seed=6, device="cuda")
+    masks = inputs.make_mask(wl)
+    tokens = inputs.make_tokens(wl, masks)
+    h0 = inputs.make_h0(w["embed"].cpu(), tokens).cuda()
+    out = []
+    for bad in (False, True):
+        x, mask, tok = h0.clone(), masks.cuda(), tokens.int().cuda()
+        if bad:
+            x[0] = float("nan")
+        ctx = binding.Context(binding.make_config(shape, 2, seq), w)
+        ctx.step(x, mask, seq, 1.0)
+        committed = torch.full((2,), -5, dtype=torch.int32, device="cuda")
+        ctx.commit(w["embed"], x, mask, tok, committed, rule=rule, threshold=0.0)
+        ctx.sync_status()
+        out.append((committed.tolist(), mask.cpu(), tok.cpu(), x.cpu()))
+    (c, m, t, x), (c2, m2, t2, x2) = out
+    assert c[0] >= 0 and c2 == [-1, c[1]]
+    assert torch.equal(m2[0], masks[0]) and torch.equal(t2[0], tokens[0].int()) and bool(x2[0].isnan().all())
+    assert torch.equal(m2[1], m[1]) and torch.equal(t2[1], t[1]) and torch.equal(x2[1], x[1])
+
+
 def test_a_host_call_that_fails_late_has_let_go_of_its_buffers():
     """The copy of the last result is refused (its buffer is registered in part) when the step is already enqueued: when the
     call comes back with its error, nothing that it enqueued runs any more, and the error is not left for the next caller."""
