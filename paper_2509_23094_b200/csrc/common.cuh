@@ -228,7 +228,9 @@ int launch_gemm_tc(const GemmArgs& g, GemmEpilogue epi, cudaStream_t st, int* st
 int gemm_tc_ctas(const GemmArgs& g, GemmEpilogue epi);         // CTAs of a launch, one per SM
 bool gemm_tc_supported(const GemmArgs& g);       // false: launch_gemm_tc would fall back to the mma.sync kernel
 // ---- two-SM tcgen05 GEMM (gemm_tc2.cu): pairs of CTAs on 256-row tiles ---------------------------
+constexpr int kPairRows = 128;                                 // rows of capacity from which on it is used
 bool gemm_tc2_supported(const GemmArgs& g);
+long long gemm_tc2_clusters(long long blocks, long long rows, int K);      // most clusters of a launch over that many blocks of 256 weight rows
 int gemm_tc2_ctas(const GemmArgs& g, GemmEpilogue epi, bool narrow_tiles = true);      // narrow_tiles: with those for 64-token tiles
 int launch_gemm_tc2(const GemmArgs& g, GemmEpilogue epi, cudaStream_t st, int* status = nullptr);
 }  // namespace d2c

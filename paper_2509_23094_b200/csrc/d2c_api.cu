@@ -66,13 +66,35 @@ static int rollout_depth(const d2c_config& c) {
 static int lm_tiles(int vocab) { return ceil_div(vocab, 128); }
 
 // The fused QKV projection leaves only Q and, after attention, the log-sum-exp in activation buffers.  Each layer uses the
-// next of kQBufs of them, so that the probabilities pass of a layer, on a stream of its own, may take longer than the layer
-// without holding up the projections of the next ones.  The last layer uses the first.
-static constexpr int kQBufs = 6;
+// next of up to six of them, so that the probabilities pass of a layer, on a stream of its own, may take longer than the layer
+// without holding up the projections of the next ones.  The last layer uses the first.  As many are carved as the rows of one
+// whole QKV buffer and of the buffers that share a place (see carve) leave room for, so that they cost no memory of their own:
+// six for as many KV heads as query heads, five for 28 and 4.
+static int q_buffers(const d2c_config& c) {
+  const size_t d = c.d_model, hq_dh = (size_t)c.n_q_heads * c.head_dim, qkv_out = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
+  const size_t stats = 6 * (size_t)lm_tiles(c.vocab), shared = stats < (size_t)c.d_ffn ? stats : (size_t)c.d_ffn;      // in elements of bf16
+  const size_t n = (qkv_out + 2 * (d < hq_dh ? d : hq_dh) + shared) / hq_dh;
+  return n < 6 ? (int)n : 6;
+}
+// Slots for parked parts: four for every cluster that the pair kernel can have at these sizes, and what the one-SM kernel may use.
+static int sk_tiles(const d2c_config& c) {
+  const int shapes[5][2] = {{(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, c.d_model}, {c.d_model, c.n_q_heads * c.head_dim},
+                            {2 * c.d_ffn, c.d_model}, {c.d_model, c.d_ffn}, {c.vocab, c.d_model}};      // {weight rows, K}
+  const long long rows = (long long)c.max_batch * c.max_seq;
+  long long most = 0;
+  for (const auto& s : shapes) {
+    const long long n = rows >= kPairRows ? gemm_tc2_clusters(ceil_div(s[0], 256), rows, s[1]) : 0;
+    most = n > most ? n : most;
+  }
+  const long long n = 4 * most < kSkMaxTiles ? 4 * most : kSkMaxTiles;
+  return n > 160 ? (int)n : 160;
+}
+// Pieces that are never live at the same time share a place: the attention output of the layers, the LM head's rows and the
+// staged h0 (read by the first kernel behind selection); the FFN's middle and the LM head's statistics.
 static size_t carve(const d2c_config& c, void* base, Buffers* out) {
   Carver w(base);
   Buffers b;
-  const size_t B = c.max_batch, L = c.max_seq, R = B * L, d = c.d_model;
+  const size_t B = c.max_batch, L = c.max_seq, R = B * L, d = c.d_model, n_q = q_buffers(c);
   const size_t hq_dh = (size_t)c.n_q_heads * c.head_dim, kv = (size_t)c.n_kv_heads * c.head_dim, qkv_out = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
   b.kcache = w.take<bf16>((size_t)c.n_layers * R * kv);
   b.vcache = w.take<bf16>((size_t)c.n_layers * R * kv);
@@ -82,18 +104,20 @@ static size_t carve(const d2c_config& c, void* base, Buffers* out) {
   b.lm_rows = w.take<int32_t>(R); b.lm_off = w.take<int32_t>(B + 1); b.slot_of_pos = w.take<int32_t>(R);
   b.rank_s = w.take<int32_t>(R); b.rank_lm = w.take<int32_t>(R); b.n_b = w.take<int32_t>(B); b.nm_b = w.take<int32_t>(B);
   b.phi = w.take<uint32_t>(L); b.rope = w.take<float2>(L * (c.head_dim / 2));
-  b.x = w.take<bf16>(R * d); b.xn = w.take<bf16>(R * d); b.qkv = w.take<bf16>(R * (qkv_out > kQBufs * hq_dh ? qkv_out : kQBufs * hq_dh));
-  b.o = w.take<bf16>(R * (size_t)c.n_q_heads * c.head_dim); b.hmid = w.take<bf16>(R * (size_t)c.d_ffn);
-  b.xm = w.take<bf16>(R * d); b.lse = w.take<float>(kQBufs * R * (size_t)c.n_q_heads);
+  b.x = w.take<bf16>(R * d); b.xn = w.take<bf16>(R * d); b.qkv = w.take<bf16>(R * (qkv_out > n_q * hq_dh ? qkv_out : n_q * hq_dh));
+  b.o = b.xm = b.h0_stage = w.take<bf16>(R * (d > hq_dh ? d : hq_dh));
+  const size_t stat = align_up(R * lm_tiles(c.vocab) * sizeof(float), 256), mid = R * (size_t)c.d_ffn * sizeof(bf16);
+  char* shared = w.take<char>(3 * stat > mid ? 3 * stat : mid);
+  b.hmid = reinterpret_cast<bf16*>(shared);
+  b.st_max = reinterpret_cast<float*>(shared); b.st_sum = reinterpret_cast<float*>(shared + stat); b.st_arg = reinterpret_cast<int32_t*>(shared + 2 * stat);
+  b.lse = w.take<float>(n_q * R * (size_t)c.n_q_heads);
   b.ssq = w.take<float>(R * (d / 32));                      // per (row, 32 columns): sum of squares of the residual stream
   b.abar = w.take<float>((size_t)rollout_depth(c) * R * L);
-  const size_t nt = lm_tiles(c.vocab);
-  b.st_max = w.take<float>(R * nt); b.st_sum = w.take<float>(R * nt); b.st_arg = w.take<int32_t>(R * nt);
   b.u0 = w.take<float>(R); b.u1 = w.take<float>(R);
   b.partial = w.take<float>((size_t)kRolloutSplit * R + (R + 3) / 4);     // partial sums + selected-flag bytes
-  b.sk_partials = w.take<float>((size_t)kSkMaxTiles * 128 * 256); b.sk_counters = w.take<int32_t>(2 * kSkMaxTiles);     // arrival and done counters
+  b.sk_partials = w.take<float>((size_t)sk_tiles(c) * 128 * 256); b.sk_counters = w.take<int32_t>(2 * kSkMaxTiles);     // arrival and done counters
   b.gemm_clocks = w.take<long long>(4);
-  b.h0_stage = w.take<bf16>(R * d); b.mask_stage = w.take<uint8_t>(R);
+  b.mask_stage = w.take<uint8_t>(R);
   b.forced_stage = w.take<int32_t>(R); b.forced_off_stage = w.take<int32_t>(B + 1);
   b.okey_stage = w.take<float>(R); b.oc_stage = w.take<float>(R); b.committed_stage = w.take<int32_t>(B);
   if (out) *out = b;
@@ -125,7 +149,7 @@ struct d2c_ctx {
   const bf16 *g_final, *w_lm;
   cudaStream_t stream;
   Buffers buf;
-  int phi_len;
+  int phi_len, q_bufs, sk_tiles;
   // Selected-row count of the previous step, which chooses between the GEMM kernels (both are correct for any
   // count, but they add fp32 partial sums in different orders).  The selection kernel writes the count into one
   // of two words of mapped host memory; the next step waits for the event recorded behind that kernel before it
@@ -212,11 +236,11 @@ static int gemm(d2c_ctx* ctx, const GemmArgs& g, GemmEpilogue epi) {
     GemmArgs g2 = g;
     g2.narrow_pairs = ctx->narrow_pairs;
     g2.max_pairs = epi == EPI_LMSTATS ? ctx->lm_pairs : ctx->max_pairs;
-    g2.sk_partials = ctx->buf.sk_partials; g2.sk_counters = ctx->buf.sk_counters; g2.sk_max_tiles = kSkMaxTiles;
+    g2.sk_partials = ctx->buf.sk_partials; g2.sk_counters = ctx->buf.sk_counters; g2.sk_max_tiles = ctx->sk_tiles;
     return launch_gemm_tc2(g2, epi, ctx->run, ctx->buf.status);
   }
   GemmArgs gs = g;
-  gs.sk_partials = ctx->buf.sk_partials; gs.sk_counters = ctx->buf.sk_counters; gs.sk_max_tiles = kSkMaxTiles;
+  gs.sk_partials = ctx->buf.sk_partials; gs.sk_counters = ctx->buf.sk_counters; gs.sk_max_tiles = ctx->sk_tiles;
   return launch_gemm_tc(gs, epi, ctx->run, ctx->buf.status);
 }
 // A CUDA runtime call inside the step: its error text goes where launcher errors go.
@@ -288,6 +312,7 @@ int d2c_create(const d2c_config* cfg, const d2c_weights* w, void* workspace, siz
   ctx->maps.resize(6 * (size_t)cfg->n_layers + 1);
   ctx->g_final = (const bf16*)w->g_final; ctx->w_lm = (const bf16*)w->w_lm;
   carve(*cfg, workspace, &ctx->buf);
+  ctx->q_bufs = q_buffers(*cfg); ctx->sk_tiles = sk_tiles(*cfg);
   {
     bool ok = cudaHostAlloc(reinterpret_cast<void**>(&ctx->hint_host[0]), 2 * sizeof(int32_t), cudaHostAllocMapped) == cudaSuccess;
     if (ok) {
@@ -558,11 +583,13 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
       D2C_TRY(ctx, launch_rmsnorm(x, nullptr, n_rows, R, d, ctx->g_attn[l], c.rms_eps, b.xn, st));
     }
     D2C_TRY(ctx, mark(ctx, PH_QKV));
-    const int qbuf = (c.n_layers - 1 - l) % kQBufs;
-    // Probabilities passes on the side stream still read their layers' Q and LSE.  Every fourth layer waits for the pass
-    // three layers back, and with it for those before: then layers l to l + 3 may write the buffers of l - 6 to l - 3.
-    const int need = fused_qkv ? l - 3 : l - 1;
-    if (abar_last >= 0 && need >= 0 && ((l & 3) == 0 || !fused_qkv))
+    const int qbuf = (c.n_layers - 1 - l) % ctx->q_bufs;
+    // Probabilities passes on the side stream still read their layers' Q and LSE.  Every fourth layer waits for those whose
+    // buffers it and the next three write: with six buffers for the pass three layers back, and with it for those before, as
+    // layers l to l + 3 write the buffers of l - 6 to l - 3.  (With fewer than four buffers every layer waits for its own.)
+    const bool by_four = fused_qkv && ctx->q_bufs >= 4;
+    const int need = by_four ? l + 3 - ctx->q_bufs : l - (fused_qkv ? ctx->q_bufs : 1);
+    if (abar_last >= 0 && need >= 0 && (!by_four || (l & 3) == 0))
       D2C_TRY(ctx, cu(cudaStreamWaitEvent(st, ctx->ev_abar[(need < abar_last ? need : abar_last) & 3], 0)));
     GemmArgs g{};
     g.A = b.xn; g.lda = d; g.W = ctx->wqkv[l]; g.bias = ctx->bqkv[l]; g.C = b.qkv; g.ldc = qkv_out;

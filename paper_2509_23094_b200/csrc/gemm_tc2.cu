@@ -35,9 +35,15 @@
 
 namespace d2c {
 // No more clusters than there are token tiles times shares of three stages, or 64-token tiles.
+static long long share_clusters(long long blocks, long long rows, int K) { return blocks * ((rows + 255) / 256) * ceil_div(ceil_div(K, 128), 3); }
+static long long narrow_clusters(long long blocks, long long rows) { return blocks * ((rows + 63) / 64); }
+long long gemm_tc2_clusters(long long blocks, long long rows, int K) {
+  const long long shares = share_clusters(blocks, rows, K), narrow = narrow_clusters(blocks, rows);
+  return narrow > shares ? narrow : shares;
+}
 int gemm_tc2_ctas(const GemmArgs& g, GemmEpilogue epi, bool narrow_tiles) {
   const long long blocks = ceil_div(g.N, epi == EPI_SWIGLU ? 128 : 256);
-  const long long shares = blocks * ceil_div(g.max_rows, 256) * ceil_div(ceil_div(g.K, 128), 3), all = blocks * ceil_div(g.max_rows, 64);
+  const long long shares = share_clusters(blocks, g.max_rows, g.K), all = narrow_clusters(blocks, g.max_rows);
   const long long narrow = g.narrow_pairs > 0 && g.narrow_pairs < all ? g.narrow_pairs : all;
   const long long most = narrow_tiles && narrow > shares ? narrow : shares;
   const int fit = g.max_pairs > 0 && g.max_pairs < sm_count_current() / 2 ? g.max_pairs : sm_count_current() / 2;
@@ -1005,7 +1011,7 @@ int launch_one(const GemmArgs& g, int* status, cudaStream_t st) {
 
 // Shapes the pair kernel takes; everything else goes to the one-SM kernel.
 bool gemm_tc2_supported(const GemmArgs& g) {
-  return g.max_rows >= 128 && g.N >= 256 && g.K % TK == 0 && (g.lda & 7) == 0 && (g.N & 1) == 0 && (g.ldc & 1) == 0 &&
+  return g.max_rows >= kPairRows && g.N >= 256 && g.K % TK == 0 && (g.lda & 7) == 0 && (g.N & 1) == 0 && (g.ldc & 1) == 0 &&
          (reinterpret_cast<uintptr_t>(g.A) & 15) == 0 && (reinterpret_cast<uintptr_t>(g.W) & 15) == 0;
 }
 

@@ -46,6 +46,17 @@ def test_workspace_bytes_and_config_validation(lib):
     assert lib.d2c_workspace_bytes(None) == 0
 
 
+# Bytes with one whole QKV buffer, every piece in a place of its own and 160 slots for parked parts: the buffers that later
+# ways of cutting the work take come out of shared places, so that a caller who filled a card with this much still fits.
+# The slots are the exception where few rows share little else: up to 160 more of 128 KB.
+@pytest.mark.parametrize("shape,batch,seq,plain,slots", [
+    (inputs.TOY, 1, 33, 21255168, 0), (inputs.TOY, 1, 128, 22484736, 0), (inputs.TOY_HD128, 2, 2048, 136514816, 160),
+    (inputs.LLADA_8B, 1, 100, 85330944, 0), (inputs.LLADA_8B, 1, 1024, 831345920, 0), (inputs.LLADA_8B, 8, 4096, 37749214464, 0),
+    (inputs.DREAM_7B, 4, 1536, 2032465152, 160), (inputs.DREAM_7B, 8, 4096, 20142050560, 0)])
+def test_workspace_does_not_grow(lib, shape, batch, seq, plain, slots):
+    assert 0 < binding.d2c_workspace_bytes(binding.make_config(shape, batch, seq)) <= plain + slots * 128 * 256 * 4
+
+
 def test_create_rejects_bad_arguments_without_a_device(lib):
     cfg = binding.make_config(inputs.TOY, 1, 128)
     handle = C.c_void_p()
