@@ -34,6 +34,12 @@
  *     into a CUDA graph from the caller's stream and replayed (the choice between
  *     kernel variants that follows an earlier step's row count is then frozen).
  *     One context per stream; a context is not re-entrant.
+ *   - What a step computes does not depend on the steps before it, but its last bits
+ *     do: the row count of the previous step (none in a capture) decides how sums are
+ *     split and whether the RMSNorms are folded into the projections.  Behind steps of
+ *     one size the same inputs and state give the same bits; behind others the results
+ *     differ within the roundings to bf16 (hidden states by up to 2e-3 of a row's norm
+ *     in one or two layers).
  *   - Return value: D2C_OK or a negative D2C_E* code; d2c_last_error() gives the
  *     text.  Nothing throws, aborts or traps.  Faults detected on the device
  *     (a bounded wait that ran out) are written to a status word that
@@ -80,7 +86,7 @@ typedef struct {
 #define D2C_FLAG_FOLDED_NORMS 16        /* fold the layers' RMSNorms into the GEMM epilogues around them (x * gain and the row's sums of
                                            squares written by the residual epilogue, the row scale applied by the next projection)
                                            instead of running them as kernels of their own; a step that expects few rows (at most 128, going
-                                           by the previous step) does so without the flag                                            */
+                                           by the previous step) does so without the flag, which moves its results by roundings       */
 
 /* Weights.  The arrays of per-layer pointers are HOST arrays of n_layers DEVICE
  * pointers; they are copied at create, the device memory is borrowed for the
@@ -147,7 +153,10 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* args, const d2c_step_out* out);
  * [batch*seq_len], row_off_host [batch+1], hidden_out_host bf16 [batch*seq_len][d] (the copy starts before the row
  * count is known, so the whole buffer may be written; rows beyond row_off_host[batch] are meaningless),
  * conf_host / pred_host [batch][seq_len] (any may be NULL).  Copies in, runs
- * d2c_step, copies out, and synchronises the stream before returning. */
+ * d2c_step and copies out; pinned buffers of up to 64 KB, and h0 and the hidden rows when the previous step left few rows to
+ * expect, are read and written in place by the step's kernels instead (a buffer that is not wholly inside one pinned
+ * allocation or registration, or does not start at a multiple of 4 bytes, 16 for rows, is copied).  The buffers are not used any more when the
+ * call returns, whatever it returns. */
 typedef struct {
   int32_t* sel_idx_host; int32_t* row_off_host; void* hidden_out_host;
   float* conf_host; int32_t* pred_host;

@@ -152,7 +152,7 @@ struct GemmArgs {
   // EPI_LMSTATS: per (row, 128-column tile) running max / sum of exp / arg-max, optional raw logits
   float* st_max; float* st_sum; int32_t* st_arg; float* logits; int n_tiles;
   // EPI_QKV_ROPE (tcgen05 kernels only): rotary embedding of Q/K and the K/V scatter into the cache fused into
-  // the QKV projection; C/ldc is the QKV activation buffer (only its Q part is written)
+  // the QKV projection; C/ldc is one of the Q buffers, a row of all query heads (ldc = q_hq * q_dh); K and V only go to the cache
   const int32_t* q_sel_idx; const int32_t* q_row_seq; const float2* q_rope; bf16* q_kc; bf16* q_vc;
   int q_cache_seq, q_hq, q_hkv, q_dh;
   // split-K scratch of the tcgen05 kernels (null: no split): sk_max_tiles partial tiles of 128 x 256 fp32

@@ -89,9 +89,9 @@ __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v,
 // rs.hist must be zero on entry and is zero again on return.
 // [vmin, vmax] bounds the members' value bits.  Digits are taken from the distance to vmin, eight bits at a time from its
 // highest on: the first pass spreads the members over up to 256 bins whatever their scale, and as soon as no more than 32 carry
-// the crossing digits, one warp places those by comparing them with each other.  (A pass takes 2500 clocks, mostly latency;
-// flat scores of 1024 positions took three or four
-// and now take one and that comparison: a step of 277 rows in two sequences 139.3 -> 135.7 us, one of 55 in 546 122.7 -> 120.7.)
+// the crossing digits, one warp places those by comparing them with each other.  (A pass takes 2500 clocks, mostly latency.
+// Flat scores of 1024 positions took three or four and now take one and that comparison: a step of 277 rows in two sequences
+// 139.3 -> 135.7 us, one of 55 in 546 122.7 -> 120.7.)
 template <typename Member, typename Weight, typename Crossed>
 __device__ __forceinline__ void take_until_crossed(const uint32_t* vb, int L, Member member, Weight weight, Crossed crossed,
                                                    uint8_t* flags, uint8_t mark, RadixScratch& rs, uint32_t vmin, uint32_t vmax) {

@@ -66,8 +66,8 @@ __device__ __forceinline__ bool meet_or_leave(bool gave_up) {
                : "=r"(any) : "n"(id), "n"(threads), "r"(mine) : "memory");
   return any != 0;
 }
-// 1 in one lane of a converged warp.  The warps that issue tcgen05 instructions run their loops with all lanes and
-// predicate only the instruction itself: under a divergent `if (lane == 0)` every descriptor word of every MMA goes
+// 1 in one lane of a converged warp.  The warps that issue the attention kernels' tcgen05 instructions run their loops with
+// all lanes and predicate only the instruction itself (the GEMMs' still run them in one lane): under a divergent `if (lane == 0)` every descriptor word of every MMA goes
 // through its own move to a uniform register first, which made an MMA cost about 58 clocks of issue.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t e;

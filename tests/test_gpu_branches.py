@@ -181,6 +181,59 @@ def test_same_step_gives_the_same_bits(seq, rows):
     ctx.sync_status()
 
 
+def test_results_behind_a_large_a_small_and_a_captured_step():
+    """The step before decides how the work is cut and, with at most 128 rows expected, that the norms ride in the projections:
+    the same inputs and state give the same bits behind steps of one size, and the same numbers within roundings behind
+    others and in a capture (which goes by none).  Two layers of four roundings to bf16 in a row: 8 * 2^-9 = 1.6e-2 of a row's
+    norm, a confidence's logit error below 3 %."""
+    shape, seq, rows = replace(inputs.TOY_HD128, name="deep", d_model=1024, d_ffn=2880, n_q_heads=8, n_kv_heads=8, vocab=4106), 701, 96
+    wl = inputs.Workload("bits", shape, 1, seq, 64, seq - 64, "all", 0, 0.0, seed=4)
+    w = inputs.make_weights(shape, seed=4, device="cuda", gain_jitter=0.05)
+    mask = inputs.make_mask(wl)
+    h0, mask = inputs.make_h0(w["embed"], inputs.make_tokens(wl, mask)).cuda(), mask.cuda()
+    conf0 = inputs.make_scores(seq, 9).view(1, seq).cuda()
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        ctx = binding.Context(binding.make_config(shape, 1, seq), w)
+        hid = torch.zeros(seq, shape.d_model, dtype=torch.bfloat16, device="cuda")
+        ctx.step(h0, mask, seq, 1.0)
+        cache = [(n, ctx.view(n).clone()) for n in ("kcache", "vcache")]
+
+        def restore():
+            for n, t in cache:
+                ctx.view(n).copy_(t)
+            ctx.view("conf", 1, seq).copy_(conf0)
+
+        def outputs():
+            ctx.sync_status()
+            assert int(ctx.view("row_off")[1]) == rows
+            return [t.clone() for t in (ctx.view("sel_idx")[:rows], hid[:rows], ctx.view("kcache"), ctx.view("vcache"),
+                                        ctx.view("conf", 1, seq), ctx.view("c", 1, seq))]
+
+        def behind(before):
+            restore()
+            ctx.step(h0, mask, before, 0.0)
+            restore()
+            ctx.step(h0, mask, rows, 0.0, hidden_out=hid)
+            return outputs()
+        few, many, few2, many2 = (behind(n) for n in (rows, 600, 40, 600))
+        restore()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            ctx.step(h0, mask, rows, 0.0, hidden_out=hid)
+        graph.replay()
+        captured = outputs()
+    assert all(torch.equal(a, b) for a, b in zip(many, many2))
+    for other in (many, few2, captured):
+        assert torch.equal(few[0], other[0])
+        for a, b in zip(few[1:4], other[1:4]):
+            assert row_rel_err(a.float().cpu().numpy(), b.float().cpu().numpy()) <= 1.6e-2
+        torch.testing.assert_close(few[4], other[4], rtol=3e-2, atol=0)
+        torch.testing.assert_close(few[5], other[5], rtol=2e-2, atol=0)
+
+
 # Top-p's crossing digits carried by 1, 31, 32 (placed by comparing them) and 33 or more members (another pass), apart by one
 # or 16 ulps, in ties of three, all equal, and with a lone far value that widens the range: the oracle's set exactly.
 @pytest.mark.parametrize("m", [1, 31, 32, 33, 300])
