@@ -532,8 +532,11 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   // Small models: the probabilities pass also goes to the side stream when its CTAs and those of any projection fit the
   // GPU together (two layers of d 512, 277 rows: 12 us a layer off the chain).
   bool small = false;
-  // Grids grow for 64-token tiles only with up to 1024 positions: with more, kernels around them want the SMs (three layers of
-  // d 256, 1500 rows: 336 us with, 317 without; 299 rows of 768 in two layers of d 512: 143 with, 155 without).
+  // Grids grow for 64-token tiles only with up to 1024 positions: with more, kernels around them (attention, whose time goes
+  // with the positions, and the probabilities beside the chain) want the SMs, whatever the rows.  Without / with, us: three
+  // layers of d 256 at 2000 positions 58 rows 242 / 242, 259 rows 263 / 275, 929 rows 320 / 404, 1668 rows 400 / 445; two of d 512
+  // 134 / 137, 156 / 156, 191 / 195, 234 / 238.  At 1100 it can go either way (497 rows 230 / 224, two layers 158 / 159), at 768
+  // with wins (299 rows in two layers of d 512: 155 / 143).
   ctx->narrow_pairs = c.n_layers > 1 && R > 1024 ? 1 : 0;
   if (!few_rows && fused_qkv) {
     AttnArgs t{};
