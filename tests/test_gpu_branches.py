@@ -84,6 +84,19 @@ def test_passes_beside_the_chain(batch, seq, p):
     np.testing.assert_allclose(a["c"].cpu().numpy(), b["c"].cpu().numpy(), rtol=2e-2)
 
 
+# Wide heads over a narrow model leave room for one (16 query and 2 KV heads), three (16 and 16) or five (8 and 2) Q buffers: a layer
+# waits for the pass whose buffer it takes, with few rows (p = 0.05) and with more, and the bits are those of one stream.
+@pytest.mark.parametrize("heads,kv,d,vocab", [(16, 2, 256, 1002), (16, 16, 256, 1002), (8, 2, 1024, 40000)])
+@pytest.mark.parametrize("p", [0.05, 0.9])
+def test_passes_beside_the_chain_with_fewer_buffers(heads, kv, d, vocab, p):
+    shape = replace(inputs.TOY_HD128, name="wide", n_layers=9, d_model=d, n_q_heads=heads, n_kv_heads=kv, d_ffn=2816, vocab=vocab)
+    got, serial = (_steps(shape, 1, 701, 100, 16, p, flags, 4) for flags in (0, 8))
+    for a, b in zip(got, serial):
+        assert a["rows"] == b["rows"]
+        for key in ("sel", "hidden", "c", "conf", "kcache"):
+            assert torch.equal(a[key], b[key]), key
+
+
 # Row counts at the edges of the token tiles (16-token units, 64-token tiles, the 128-row regime, 256-token tiles, several
 # tiles) on the pair GEMM with all of its epilogues, on the forward that shares keys between CTAs and on the probabilities
 # kernel, against the portable kernels.  128 and 150 positions are the smallest contexts the pair GEMM takes, 2100 keys let four
