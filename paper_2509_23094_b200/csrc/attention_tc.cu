@@ -282,17 +282,12 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       const float sc = kLog2e * rsqrtf((float)ADH);
       float m_used = -INFINITY, l = 0.f;
       bool ok = true;
-      const bool dead = lrow - lane >= nrows;                       // none of the warp's rows is live: it only keeps step
       for (int j = 0; j < T && ok; ++j) {
         const int sp = dbuf ? (j & 1) : q;                          // S/P buffer of this tile
         const uint32_t ts = tm + sp * 256 + lane_base;
         // a wait that gave up ends the loop for the whole warp: the tcgen05.ld / st below are warp-collective
         if (!__all_sync(0xffffffffu, mbar_wait(B(7 + sp), (dbuf ? (j >> 1) : j) & 1, abortp, status, 18))) { ok = false; break; }
         tc_fence_after();
-        if (dead) {
-          if (lane == 0) { mbar_arrive(B(9 + sp)); mbar_arrive(B(13 + sp)); }
-          continue;
-        }
         const int key0 = (first + j) * AKEYS;
         const bool full = key0 + AKEYS <= L;
         uint32_t sv[4][32];                                         // the whole score row of this thread
@@ -402,6 +397,9 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         for (int t = 0; t < 4; ++t) { float lo, hi; unpack2(rs2[t], lo, hi); rs4[t] = lo + hi; }
         l += (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
       }
+      // (A warp without live rows goes all the way with the others: one that skipped the wait above passed this one a phase early, and
+      // was no faster: 976 rows of four sequences x 1536 keys 101.2 -> 100.4 us, 300 of five x 3071 139.9 -> 139.1, 147 of four x 1187
+      // 27.0 -> 27.3.)
       if (ok) ok = __all_sync(0xffffffffu, mbar_wait(B(11 + q), (T - 1) & 1, abortp, status, 19));
       tc_fence_after();
       if (kSplit && ok) {
@@ -418,7 +416,7 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                          "r"(v[4 * t]), "r"(v[4 * t + 1]), "r"(v[4 * t + 2]), "r"(v[4 * t + 3]) : "memory");
         }
         asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(sK(0) + (uint32_t)lrow * 8u), "f"(m_used), "f"(l) : "memory");
-      } else if (ok && !dead) {
+      } else if (ok) {
         // Through this warp's part of its Q tile, which every MMA has read: a row's 16-byte pieces, swizzled, go in by rows and
         // come out as whole rows.  (Each thread storing its own row, 16 bytes at a time, took 1.9 us.)
         const bool row_ok = lrow < nrows;
