@@ -73,9 +73,9 @@ constexpr float kRescaleStep = 8.f;
 constexpr int kMaxSplits = 4;
 // Of a tile's 128 keys, those whose probabilities are handed over first.  The products of the others and the next scores are what a
 // query tile waits for: 3240 clocks a pair of score tiles with 64 first, of which the special function unit takes 2048 and the tensor
-// cores as many.  With 96, us (forward alone, before / after this and the stores below): 976 rows of four sequences x 1536 keys x 28
-// heads 109.9 / 101.5, 797 x 797 x 32 20.7 / 19.9, 147 of four x 1187 x 28 28.5 / 27.0, 300 of five x 3071 x 32 141.1 / 140.0; one query
-// tile a CTA (489 x 768 x 32) 12.8 / 13.2.
+// cores as many.  Forward alone, us, with 32 / 64 / 96 first: 976 rows of four sequences x 1536 keys x 28 heads 105.4 / 103.8 / 100.2,
+// 797 x 797 x 32 20.5 / 20.3 / 19.6, 147 of four x 1187 x 28 28.3 / 28.2 / 27.3, 300 of five x 3071 x 32 143.4 / 141.9 / 138.3; one
+// query tile a CTA (489 x 768 x 32) 13.0 / 12.8 / 12.8.
 constexpr int kFirstKeys = 96;
 
 // Packed pairs of fp32 for Blackwell's two-wide FMA-pipe instructions: one issue slot for two elements.
@@ -111,7 +111,6 @@ template <bool kSplit>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const AttnTcParams p) {
-  if (threadIdx.x == 0) { prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV); }      // (101.5 us; 112 without)
   pdl_prologue();
   const AttnArgs& a = p.a;
   // split: the row tile is the slowest index, so that the live ones start first (beyond them CTAs only find nothing to do)
@@ -313,7 +312,7 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         // scale-and-subtract and the row sums run two elements per instruction (fma / add .f32x2)
         unsigned long long rs2[4];                                  // packed pairs of partial row sums
         const unsigned long long sc2 = pack2(sc, sc);
-        uint32_t pk[2][8];
+        uint32_t pk[AKEYS / 32][16];
         // probabilities of the keys [16 b0, 16 b1), rounded to bf16, in batches of 16: a batch is summed and rounded behind the
         // next one's exponentials, so that nothing waits for a result of the special function unit
         auto some_keys = [&](auto b0_, auto b1_, bool with_max) {
@@ -338,13 +337,7 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
                 rs2[i & 3] = add2(rs2[i & 3], pack2(pp[d & 1][2 * i], pp[d & 1][2 * i + 1]));
-                pk[d & 1][i] = pack_bf16(pp[d & 1][2 * i], pp[d & 1][2 * i + 1]);
-              }
-              if (d & 1) {                                          // 32 keys' worth
-                uint32_t w[16];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) { w[i] = pk[0][i]; w[8 + i] = pk[1][i]; }
-                tmem_st16(ts + (d >> 1) * 16, w);
+                pk[d >> 1][(d & 1) * 8 + i] = pack_bf16(pp[d & 1][2 * i], pp[d & 1][2 * i + 1]);
               }
             }
           }
@@ -379,10 +372,14 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
           zero_sums();
           some_keys(kBegin, kMid, false);
         }
-        // written back as bf16 over the scores: the product with V starts on the first keys while the others' are worked out
+        // written back as bf16 over the scores: the product with V starts on the first keys while the others' are worked out.  (Not
+        // stored among the exponentials: the kernel then spills, 20 to 24 bytes by chance of what stands elsewhere in it, and is up to
+        // 10 % slower: 976 rows of four sequences x 1536 keys 100 us, 101 or 112 that way.)
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           if (hf == 1) some_keys(kMid, kEnd, false);
+#pragma unroll
+          for (int c = hf ? kFirstKeys / 32 : 0; c < (hf ? AKEYS : kFirstKeys) / 32; ++c) tmem_st16(ts + c * 16, pk[c]);
           tmem_st_wait();
           // Behind the loop the last product is waited for, and a parity wait only tells a phase from the one before it.  The
           // last scores do not wait for the product before the last (its V may come in late), so that one is waited for
