@@ -458,15 +458,25 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   const Buffers& b = ctx->buf;
   // critical path on `st`, probabilities + rollout on `side` (the same stream while profiling or when serial)
   const int B = a->batch, L = a->seq_len, R = B * L, d = c.d_model;
-  bool fills = false;                                  // the LM head's product takes all SMs
+  // Whether a product's weights alone give all SMs work, with one tile of tokens and whichever kernel takes it.  (By the tiles of all
+  // tokens that there is room for the smallest models' products would, at lengths where most of those CTAs find no rows; called
+  // large, they lose: one layer of d 256, us, 1200 positions 106 / 120, all rows 93 / 112, 2048 positions 149 / 176; two of d 512 at
+  // 2 x 2048 303 / 310, all rows 319 / 332, 103 rows of 2048 positions 131 / 150.  The other way: two of d 512, all of 1200 rows, 180 / 174.)
+  auto takes_all = [&](int n, int k, GemmEpilogue epi) {
+    GemmArgs t{};
+    t.max_rows = R < 256 ? R : 256; t.N = n; t.K = k;
+    return gemm_tc2_ctas(t, epi, false) >= sm_count_current() - 1;
+  };
+  const bool lm_takes_all = takes_all(c.vocab, d, EPI_LMSTATS), layers_take_all = takes_all(c.d_ffn, d, EPI_SWIGLU);
+  bool fills = false;                                  // the LM head takes all SMs, and can be told to leave some
   {
     GemmArgs t{};
     t.A = b.xm; t.W = ctx->w_lm; t.max_rows = R; t.N = c.vocab; t.K = t.lda = d;
-    fills = !(c.flags & (D2C_FLAG_PORTABLE_GEMM | D2C_FLAG_ONE_SM_GEMM)) && gemm_tc2_supported(t) && gemm_tc2_ctas(t, EPI_LMSTATS) >= sm_count_current() - 1;
+    fills = lm_takes_all && !(c.flags & (D2C_FLAG_PORTABLE_GEMM | D2C_FLAG_ONE_SM_GEMM)) && gemm_tc2_supported(t);
   }
   // Models whose products leave SMs free need no priority over the passes beside them: their chain stays on the caller's stream,
   // without the two events between streams (one layer of d 256 at 94 rows 56.4 -> 53.4 us, two of d 512 at 299 rows 121.1 -> 119.6).
-  const bool overlap = ctx->work_stream != nullptr && !ctx->prof, hop = overlap && fills;
+  const bool overlap = ctx->work_stream != nullptr && !ctx->prof, hop = overlap && (lm_takes_all || layers_take_all);
   cudaStream_t st = hop ? ctx->work_stream : ctx->stream;
   cudaStream_t side = overlap ? ctx->side_stream : st;
   ctx->run = st;
@@ -475,9 +485,9 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     D2C_TRY(ctx, cu(cudaStreamWaitEvent(st, ctx->ev_in, 0)));
   }
   // The probabilities pass of a layer goes to the side stream when its CTAs cannot hold up the projections that follow:
-  // with few rows or in small models, for a small single layer (it then overlaps the LM head), and on SM pairs that the projections
-  // leave alone.  Otherwise a statically scheduled GEMM whose CTAs start late behind side-stream CTAs loses more than the
-  // overlap gains (measured at 488 rows x 32 layers: +5 %).
+  // with few rows or in small models, for a single layer whose products leave SMs free (it then overlaps the LM head), and on SM
+  // pairs that the projections leave alone.  Otherwise a statically scheduled GEMM whose CTAs start late behind side-stream CTAs
+  // loses more than the overlap gains (measured at 488 rows x 32 layers: +5 %).
   // regime of this step: the row count of the previous step, read behind that step's selection kernel
   const bool capturing = stream_captures(ctx), track = ctx->hint_host[0] != nullptr && !capturing;
   const int slot = (int)(ctx->step_no & 1);
@@ -586,9 +596,9 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     const int free_pairs = (sm_count_current() - attention_abar_sms(t)) / 2;
     small = c.n_layers > 1 && most <= 2 * free_pairs;
     if (small) ctx->max_pairs = free_pairs;
-    // A small single layer's pass runs beside its products in any case: 64-token tiles only spread over the SMs it leaves (one layer of
-    // d 256, 1200 rows: 98 us, over all SMs 121, which then wait for the pass).
-    if (c.n_layers == 1 && !fills) ctx->narrow_pairs = free_pairs > 1 ? free_pairs : 1;
+    // The pass of a single layer whose products leave SMs free runs beside them in any case: 64-token tiles only spread over the SMs
+    // it leaves (one layer of d 256, 1200 rows: 93 us, over all SMs 113, which then wait for the pass).
+    if (c.n_layers == 1 && !layers_take_all) ctx->narrow_pairs = free_pairs > 1 ? free_pairs : 1;
   }
   // Large models, more rows: the pass is short (489 rows x 768 keys: 17 us) but takes that on the whole GPU, mostly latency.  A
   // few SM pairs do it in the time of a layer, and the layer's other kernels lose less by those than the pass took between
@@ -603,10 +613,12 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     if (attention_tc_supported(t)) abar_pairs = attention_abar_pairs(t, 40.f + flops / 1.1e9f);      // 1.1 PFLOP/s and 40 us of small kernels
     if (abar_pairs > 0) ctx->max_pairs = sm_count_current() / 2 - abar_pairs;
   }
-  // A single large layer's pass stays on the chain: beside it it gets SMs in the gaps between launches, where it holds up the statically
-  // scheduled CTAs behind it, and ends after the LM head.  One layer beside / on the chain, us: 831 rows x 1024 positions 561 / 553, 797 x 797
-  // 567 / 552, 588 rows of four sequences x 1187 613 / 587, 1499 of five x 3071 1230 / 1140.
-  const bool abar_aside = overlap && ((c.n_layers == 1 && !fills) || few_rows || small || abar_pairs > 0);
+  // A single layer's pass stays on the chain where the layer's products take all SMs: beside them it gets SMs in the gaps between launches,
+  // where it holds up the statically scheduled CTAs behind it, and ends after the LM head.  One layer beside / on the chain, us: d 4096,
+  // 831 rows x 1024 positions 561 / 553, 797 x 797 567 / 552, 588 rows of four sequences x 1187 613 / 587, 1499 of five x 3071 1230 / 1140.
+  // An LM head of that size alone is no reason: d 768 and 16000 words, 2000 rows of four sequences 167 / 176, 301 rows 87 / 96; d 1536 and
+  // 50000, 2048 positions 180 / 207; all of 2048 rows at d 768 256 / 245.
+  const bool abar_aside = overlap && ((c.n_layers == 1 && !layers_take_all) || few_rows || small || abar_pairs > 0);
   // The launches of the pair kernel: with the SM pairs that the layers leave to the passes beside them and, where the passes end
   // before the layers do, with all.
   ctx->plan.n = 0;
@@ -735,8 +747,8 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     D2C_TRY(ctx, gemm(ctx, gd, EPI_RESIDUAL));
     if (aside) {
       // The host needs longer for these calls than small kernels run, so the chain's came first: those of this layer, behind the
-      // last one also the LM head's, unless that would take all SMs.
-      if (l == c.n_layers - 1 && !fills) { last_pass = at; last_rollout = rollout_here; pass_left = true; continue; }
+      // last one also the LM head's, unless that takes all SMs.
+      if (l == c.n_layers - 1 && !lm_takes_all) { last_pass = at; last_rollout = rollout_here; pass_left = true; continue; }
       D2C_TRY(ctx, cu(cudaStreamWaitEvent(side, ctx->ev_fwd, 0)));
       D2C_TRY(ctx, launch_attention(at, side));
       D2C_TRY(ctx, cu(cudaEventRecord(ctx->ev_abar[l & 3], side)));
