@@ -14,6 +14,7 @@ namespace d2c {
 namespace {
 
 constexpr int QT = 64, KT = 64, ATHREADS = 128;
+constexpr int kSmemSm = 228 * 1024;               // shared memory of an SM
 constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes) {
@@ -249,14 +250,21 @@ __global__ void __launch_bounds__(ATHREADS) attn_abar_kernel(AttnArgs a) {
 
 template <int DH>
 int launch_dh(const AttnArgs& a, cudaStream_t st) {
-  const int smem_fwd = QT * DH * 2 + 4 * KT * DH * 2, smem_ab = 4 * KT * DH * 2;
+  const int tiles_fwd = QT * DH * 2 + 4 * KT * DH * 2, smem_ab = 4 * KT * DH * 2;
   static PerDevice attr_set;
   if (attr_set.first()) {
-    D2C_CUDA_OK(cudaFuncSetAttribute(attn_fwd_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_fwd));
+    D2C_CUDA_OK(cudaFuncSetAttribute(attn_fwd_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemSm / 2));
     D2C_CUDA_OK(cudaFuncSetAttribute(attn_abar_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_ab));
   }
   const int qtiles = ceil_div(a.max_rows_per_seq, QT);
   if (a.which != 2) {
+    // The forward's CTAs come in while the kernels before it still hold SMs, and crowd on the others: each asks for so much shared
+    // memory that no SM takes more of them than its share of the grid, and the rest wait for theirs.  us, without / with: three layers
+    // of d 256, 2048 rows 422 / 360 (81 / 64 a launch of 128 CTAs), 4096 of two sequences 555 / 506, 1503 of three sequences 222 / 212;
+    // one layer, 1400 rows of 2048 positions 147 / 136, 4096 rows 198 / 174; three layers, 206 rows of two sequences 271 / 284.  From
+    // five CTAs an SM on they fill the SMs by themselves.
+    const int per_sm = ceil_div(qtiles * a.hq * a.batch, sm_count_current()), share = kSmemSm / (per_sm + 1);
+    const int smem_fwd = tiles_fwd > share ? tiles_fwd : share;
     D2C_LAUNCH((attn_fwd_kernel<DH>), dim3(qtiles, a.hq, a.batch), ATHREADS, smem_fwd, st, a);
   }
   if (a.abar && a.which != 1) {
