@@ -651,7 +651,7 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     return rc;
   };
   AttnArgs last_pass{};                                // the last layer's pass, if it is enqueued behind the LM head
-  bool pass_left = false, last_rollout = false;
+  bool pass_left = false;
   for (int l = 0; l < c.n_layers; ++l) {
     if (out && out->layer_in) {
       cudaError_t e = cudaMemcpyAsync(static_cast<bf16*>(out->layer_in) + (size_t)l * R * d, x, (size_t)R * d * sizeof(bf16),
@@ -748,7 +748,7 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     if (aside) {
       // The host needs longer for these calls than small kernels run, so the chain's came first: those of this layer, behind the
       // last one also the LM head's, unless that takes all SMs.
-      if (l == c.n_layers - 1 && !lm_takes_all) { last_pass = at; last_rollout = rollout_here; pass_left = true; continue; }
+      if (l == c.n_layers - 1 && !lm_takes_all) { last_pass = at; pass_left = true; continue; }
       D2C_TRY(ctx, cu(cudaStreamWaitEvent(side, ctx->ev_fwd, 0)));
       D2C_TRY(ctx, launch_attention(at, side));
       D2C_TRY(ctx, cu(cudaEventRecord(ctx->ev_abar[l & 3], side)));
@@ -802,7 +802,7 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   if (pass_left) {
     D2C_TRY(ctx, cu(cudaStreamWaitEvent(side, ctx->ev_fwd, 0)));
     D2C_TRY(ctx, launch_attention(last_pass, side));
-    D2C_TRY(ctx, last_rollout ? rollout() : cu(cudaEventRecord(ctx->ev_side, side)));
+    D2C_TRY(ctx, rollout());                           // (it is put off itself only where the LM head takes all SMs)
   }
   if (!rollout_done) return fail(ctx, D2C_EINVAL, "d2c_step: no layer produced attention probabilities");
   if (overlap) D2C_TRY(ctx, cu(cudaStreamWaitEvent(st, ctx->ev_side, 0)));
