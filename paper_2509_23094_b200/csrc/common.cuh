@@ -161,9 +161,9 @@ struct GemmArgs {
   // the QKV projection; C/ldc is one of the Q buffers, a row of all query heads (ldc = q_hq * q_dh); K and V only go to the cache
   const int32_t* q_sel_idx; const int32_t* q_row_seq; const float2* q_rope; bf16* q_kc; bf16* q_vc;
   int q_cache_seq, q_hq, q_hkv, q_dh;
-  // split-K scratch of the tcgen05 kernels (null: no split): sk_max_tiles partial tiles of 128 x 256 fp32
-  // and twice as many zero-initialised counters
-  // (pair kernel: kPairCounters arrival counters, and those that the launch clears)
+  // split-K scratch of the tcgen05 kernels (null: no split): sk_max_tiles partial tiles of 128 x 256 fp32 and counters that are zero
+  // when the launch starts.  One-SM kernel: twice as many, put back at each meeting.  Pair kernel: kPairCounters, left as they are
+  // for the next launch to clear, and in sk_clear those of the launch before, which this one clears (null: none)
   float* sk_partials; int32_t* sk_counters; int sk_max_tiles; int32_t* sk_clear;
   // RMSNorm folded into the GEMMs around it (tcgen05 kernels).  A residual epilogue that is given nx_out also writes
   // nx_out[row][col] = bf16(x_new[row][col] * nx_gain[col]) (same leading dimension as C) and, per (row, 32-column

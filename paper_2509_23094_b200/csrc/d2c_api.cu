@@ -639,9 +639,10 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     ctx->max_pairs = pairs;
   }
   D2C_TRY(ctx, mark(ctx, PH_GATHER));
-  // The projections that share items leave the meeting's counters at zero, unless one of them gave up a wait.  What such a
-  // step left would let the next one add parts of another launch, so every step starts with cleared counters: in this
-  // kernel, which no GEMM overlaps that has come past its wait (in the selection kernel it took 0.3 us of the smallest step).
+  // Every step starts with cleared meeting counters, whatever the one before left in them: the one-SM kernel puts its own back at each
+  // meeting, unless a wait gave up, and the pair kernel's are cleared by the launch after (the last one's by lm_reduce).  What was left
+  // would let a launch add parts of another.  In this kernel, which no GEMM overlaps that has come past its wait (in the selection
+  // kernel it took 0.3 us of the smallest step).
   D2C_TRY(ctx, launch_gather_norm((const bf16*)a->h0, b.sel_idx, b.row_seq, n_rows, R, L, d, ctx->g_attn[0], c.rms_eps, x, b.xn,
                                   b.sk_counters, kCounters, ctx->plan, st));
   auto rollout = [&]() {

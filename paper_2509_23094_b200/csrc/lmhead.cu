@@ -14,6 +14,8 @@ lm_reduce_kernel(const float* __restrict__ st_max, const float* __restrict__ st_
                  const int32_t* __restrict__ row_seq, int seq_len, float* __restrict__ conf,
                  int32_t* __restrict__ pred, const CopyOut copies, int32_t* __restrict__ clear, int n_clear) {
   pdl_prologue();
+  // (the meeting counters of the step's last product: no launch needs it, as every step clears them at its start, but a step that ran
+  // through leaves all of them at zero, and a test reads in them that it did)
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i < n_clear; i += 256) clear[i] = 0;
   __shared__ float s_mx[8], s_sum[8];

@@ -87,8 +87,10 @@ def test_counts_left_by_a_wait_that_gave_up_do_not_reach_the_next_step():
     h0, mask = inputs.make_h0(w["embed"].cpu(), inputs.make_tokens(wl, mask)).cuda(), mask.cuda()
     conf0 = inputs.make_scores(seq, 7).view(1, seq).cuda()
     ctx = binding.Context(binding.make_config(shape, 1, seq), w)
-    n = 2 * 320                                                     # arrival and done counters, right before gemm_clocks
+    # right before gemm_clocks: arrival and done counters of the one-SM kernel, and two sets of arrival counters of the pair kernel
+    n = 2 * 320 + 2 * 160
     counters = ctx._view(ctx.state.gemm_clocks - 4 * n, n, torch.int32)
+    sets = {"one-SM": counters[:640], "pair, first set": counters[640:800], "pair, second set": counters[800:]}
     hid = torch.zeros(seq, shape.d_model, dtype=torch.bfloat16, device="cuda")
     ctx.step(h0, mask, seq, 1.0)
     for rows in (257, 96):                                          # shared between clusters with many and with few rows
@@ -100,7 +102,8 @@ def test_counts_left_by_a_wait_that_gave_up_do_not_reach_the_next_step():
             hid.zero_()
             ctx.step(h0, mask, rows, 0.0, hidden_out=hid)
             ctx.sync_status()
-            assert not counters.any()
+            for name, part in sets.items():
+                assert not part.any(), name
             runs.append([hid.clone(), ctx.view("kcache").clone(), ctx.view("conf").clone(), ctx.view("c").clone()])
         for other in runs[2:]:                                      # (the first step expects other rows than it finds)
             assert all(torch.equal(a, b) for a, b in zip(other, runs[1]))
