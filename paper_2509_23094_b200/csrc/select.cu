@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
   __shared__ RadixScratch rsc;
   __shared__ unsigned long long mlist[kRankMax];               // stage-1 members: position, then (key bits << 32 | ~position)
   __shared__ int warp_buf32[32];
-  __shared__ int s_total32, s_nm, s_nc;
+  __shared__ int s_total32, s_nm, s_known, s_listed;
   __shared__ unsigned long long s_mass;
   __shared__ uint32_t s_lo, s_hi;
   __shared__ uint32_t s_phi[kPhiMax];                          // the non-zero head of the phi table (window +-65 at sigma 10)
@@ -250,14 +250,16 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
   }
   for (int r = tid; r < min(a.phi_len, kPhiMax); r += kSelThreads) s_phi[r] = a.phi_q30[r];
   for (int i = tid; i < 3 * 256; i += kSelThreads) (&rsc.hist[0][0])[i] = 0;
-  if (tid == 0) { s_nm = 0; s_nc = 0; s_mass = 0; s_lo = 0xFFFFFFFFu; s_hi = 0u; }
+  if (tid == 0) { s_nm = 0; s_known = 0; s_listed = 0; s_mass = 0; s_lo = 0xFFFFFFFFu; s_hi = 0u; }
   __syncthreads();
   if (tid < n_forced) first_forced = a.forced[f0 + tid];
 
-  // ---- the set stage 1 ranks: masked positions inside the block, listed in any order ----
+  // ---- the set stage 1 ranks: masked positions inside the block, listed in any order; known positions are counted ----
+  int known = 0;
   for (int base = 0; base < L; base += kSelThreads) {
     const int i = base + tid;
     const bool m1 = i < L && smask[i] && i >= blk_lo && i < blk_hi;
+    known += __popc(__ballot_sync(0xffffffffu, i < L && !smask[i]));
     if (i < L) { in1[i] = m1 ? 1 : 0; if (!m1) key_out[i] = 0.f; }
     const unsigned act = __ballot_sync(0xffffffffu, m1);
     if (act) {
@@ -268,8 +270,9 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
       if (m1 && slot < kRankMax) mlist[slot] = (unsigned long long)i;
     }
   }
+  if (lane == 0) atomicAdd(&s_known, known);
   __syncthreads();
-  const int nm = s_nm;
+  const int nm = s_nm, take = min(max(a.k, 0), nm);
 
   // ---- keys (Eq. 3-4): D(i) as an exact integer sum over the window, key = fp32(D) * confidence ----
   auto known_at = [&](int i, int r) {
@@ -325,7 +328,6 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
 
   // ---- stage 1: the k largest keys of the set, lower position first among equal keys ----
   {
-    const int take = min(max(a.k, 0), nm);
     if (take == nm) {
       for (int i = tid; i < L; i += kSelThreads)
         if (in1[i]) flags[i] = F_SEL | F_MSTAR;
@@ -360,21 +362,19 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
     auto mass = [](uint32_t bits) { return (unsigned long long)__double2ull_rd((double)__uint_as_float(bits) * 4294967296.0); };
     unsigned long long local = 0;
     uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-    // (the list of the candidates, in any order, for the direct sums below; stage 1 is done with its own)
+    // Few candidates are listed, in any order, for the direct sums below (stage 1 is done with its list).  Only they: listing 500 to
+    // 1500, of which none is looked at, took up to 1 us of a step.
     unsigned long long *ckey = mlist, *cmass = mlist + kSumMax;
-    for (int base = 0; base < L; base += kSelThreads) {
-      const int j = base + tid;
-      const bool is = j < L && cand(j);
-      const unsigned long long w = is ? mass(cb[j]) : 0ull;
-      if (is) { local += w; lo = min(lo, cb[j]); hi = max(hi, cb[j]); }
-      const unsigned act = __ballot_sync(0xffffffffu, is);
-      if (act) {
-        int slot = 0;
-        if (lane == __ffs(act) - 1) slot = atomicAdd(&s_nc, __popc(act));
-        slot = __shfl_sync(0xffffffffu, slot, __ffs(act) - 1) + __popc(act & ((1u << lane) - 1u));
-        if (is && slot < kSumMax) { ckey[slot] = ((unsigned long long)cb[j] << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)j); cmass[slot] = w; }
+    const int nc = mode1 ? L - take : s_known;
+    for (int j = tid; j < L; j += kSelThreads)
+      if (cand(j)) {
+        const unsigned long long w = mass(cb[j]);
+        local += w; lo = min(lo, cb[j]); hi = max(hi, cb[j]);
+        if (nc <= kSumMax) {
+          const int slot = atomicAdd(&s_listed, 1);
+          ckey[slot] = ((unsigned long long)cb[j] << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)j); cmass[slot] = w;
+        }
       }
-    }
     for (int o = 16; o > 0; o >>= 1) local += shfl_xor_u64(local, o);
     lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi);
     if (lane == 0) {
@@ -402,10 +402,10 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
         T = hi_t;
       }
     }
-    const int nc = s_nc;
     if (nc <= kSumMax) {
-      // few candidates: the mass before each of them, a group of tpe lanes (a power of two, inside one warp) to a candidate (94 rows
-      // of 128 positions: a step 53.4 -> 52.4 us; with 243 candidates the search by digits is faster, 119.6 and 121.2)
+      // few candidates: the mass before each of them, a group of tpe lanes (a power of two, inside one warp) to a candidate.  A step of
+      // the smallest model, us, this way / by digits: 96 candidates 53.2 / 53.9, 120 57.6 / 58.2, 128 57.4 / 57.7, 150 59.3 / 59.2, 180
+      // 60.0 / 60.0, 210 62.3 / 61.4, 300 68.1 / 64.3.
       int tpe = 1;
       while (tpe < 32 && 2 * tpe * nc <= kSelThreads) tpe <<= 1;
       const int sub = tid & (tpe - 1), groups = kSelThreads / tpe;
