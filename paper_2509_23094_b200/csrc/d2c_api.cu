@@ -520,7 +520,10 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   r.spread = fills && !rollout_late;
   // With few rows (192 are a tile of tokens that the weights still bound) the LM head leaves eight SMs to that and to the rows that
   // a host call gets from a kernel.  (Where it took all SMs, those left behind it, and the kernels after it, whose start waits for
-  // every write under way to the host, came 17 us later: one layer called with host buffers 382 -> 370 us.)
+  // every write under way to the host, came 17 us later: one layer called with host buffers 382 -> 370 us.)  One layer without / with
+  // the room, us: 32 rows in the LM head 523 / 515, 64 337 / 335 and 546 / 535, 128 364 / 359 and (in four sequences) 469 / 461, 192
+  // 490 / 504 and 1419 / 1389, 384 680 / 698, 512 803 / 819.  The rollout beside it or where it could begin: no difference up to 12 MB
+  // but for 1530 rows of 2048 positions, 823 / 880; four layers, 69 MB 3219 / 3115, 94 MB 7221 / 7116.
   const bool lm_room = fills && c.stage2_candidates == 0 && (long long)B * a->k <= 192;
   const float rollout_mb = 4e-6f * r.n_layers * (float)(expect_rows < R ? expect_rows : R) * (float)L;
   const bool spread_late = r.spread && lm_room && rollout_mb <= 32.f;

@@ -552,7 +552,7 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // Launches take turns with two sets of meeting counters: this one clears the one before it, which is complete.  (Put back by the
     // last reader of each item, they cost the launch's end a barrier and an atomic's way to the L2 and back:
-    // 32 layers at 80 rows 3854 -> 3797 us, 28 at 588 rows 9180 -> 9000.)
+    // 32 layers at 80 rows 3870 -> 3820 us, 28 at 588 rows 9200 -> 9100.)
     if (g.sk_clear && blockIdx.x == 0)
       for (int i = lane; i < kPairCounters; i += 32) g.sk_clear[i] = 0;
     if (g.clock_probe && blockIdx.x == 0 && lane == 0) { g.clock_probe[0] = clock64(); g.clock_probe[1] = global_timer_ns(); }
@@ -569,8 +569,8 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (even CTA only)
     // The whole warp runs the loop and one lane's instructions take effect (see elect_one).  Under `if (lane == 0)` an MMA cost
-    // about 58 clocks of issue, what the tensor cores need for 112 tokens: 32 layers at 80 rows 4052 -> 3941 us, two of d 512 at
-    // 299 rows 133.7 -> 125.8, one of d 256 at 94 rows 59.4 -> 57.4, 32 at 797 rows 12240 -> 12080.
+    // about 58 clocks of issue, what the tensor cores need for 112 tokens: 32 layers at 80 rows 4095 -> 3985 us, two of d 512 at
+    // 299 rows 133.7 -> 125.8, one of d 256 at 94 rows 59.2 -> 57.4.
     if (leader) {
       const uint32_t el = elect_one();
       uint32_t tcount = 0;

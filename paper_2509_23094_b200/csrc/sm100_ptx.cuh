@@ -43,8 +43,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
                                           long long limit = kWaitCycles) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
-  // (up to 20 us at a time: warps that ask again and again cost the steps at the power cap 1 to 2 %, 28 layers at 3904 rows, four at
-  // 23043, and the others their issue slots)
+  // (up to 20 us at a time: warps that ask again and again take issue slots from the others: two layers of d 512 at 299 rows 118.5 ->
+  // 117.6 us, one of d 256 at 94 rows 51.3 -> 51.0; the steps at the power cap differ by less than their runs do)
   for (;;) {
     if (mbar_try_wait_for(bar, parity, 20000u)) return true;
     if (*abort_flag) return false;
