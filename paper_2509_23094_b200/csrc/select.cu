@@ -356,6 +356,8 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
   }
 
   // ---- stage 2: top-p over the candidates by influence score ----
+  // (The loops from here on are hardly unrolled: a step's weights drive these instructions out of the caches, and what is not unrolled need
+  // not come back.  Three sequences of 701 positions 91.2 -> 90.4 us, 94 rows of 128 59.7 -> 58.3 and 105.8 -> 105.1.)
   if (a.p > 0.f) {
     const bool mode1 = a.stage2_candidates != 0;
     auto cand = [&](int j) { return mode1 ? (flags[j] & F_MSTAR) == 0 : smask[j] == 0; };
@@ -366,6 +368,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
     // 1500, of which none is looked at, took up to 1 us of a step.
     unsigned long long *ckey = mlist, *cmass = mlist + kSumMax;
     const int nc = mode1 ? L - take : s_known;
+#pragma unroll 1
     for (int j = tid; j < L; j += kSelThreads)
       if (cand(j)) {
         const unsigned long long w = mass(cb[j]);
@@ -414,6 +417,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
         const unsigned long long mine = e < nc ? ckey[e] : 0ull;
         unsigned long long before = 0;
         if (e < nc)
+#pragma unroll 2
           for (int f = sub; f < nc; f += tpe) before += ckey[f] > mine ? cmass[f] : 0ull;
         for (int o = 1; o < tpe; o <<= 1) before += shfl_xor_u64(before, o);
         if (e < nc && sub == 0 && before < T) flags[0xFFFFFFFFu - (uint32_t)(mine & 0xFFFFFFFFull)] |= F_SEL;
@@ -426,6 +430,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
   }
 
   // ---- forced rows ----
+#pragma unroll 1
   for (int f = tid; f < n_forced; f += kSelThreads) {
     const int pos = f == tid ? first_forced : a.forced[f0 + f];
     if (pos >= 0 && pos < L) flags[pos] = flags[pos] | F_SEL;   // duplicates write the same value
@@ -437,11 +442,13 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
     const int per = (L + kSelThreads - 1) / kSelThreads;
     const int j0 = tid * per;
     int local = 0;                                     // low 16 bits: selected, high 16: selected & masked
+#pragma unroll 1
     for (int e = 0; e < per; ++e) {
       const int j = j0 + e;
       if (j < L && (flags[j] & F_SEL)) local += 1 + (smask[j] ? (1 << 16) : 0);
     }
     int excl = block_exclusive_scan<int>(local, warp_buf32, &s_total32);
+#pragma unroll 1
     for (int e = 0; e < per; ++e) {
       const int j = j0 + e;
       if (j >= L) break;
@@ -455,6 +462,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a) {
     }
     __syncthreads();
     // written position by position: neighbouring threads, neighbouring words
+#pragma unroll 1
     for (int j = tid; j < L; j += kSelThreads) {
       const uint32_t r = kb[j];
       const int rs = r == 0xFFFFFFFFu ? -1 : (int)(r & 0xFFFFu), rl = rs < 0 || (r >> 16) == 0xFFFFu ? -1 : (int)(r >> 16);
