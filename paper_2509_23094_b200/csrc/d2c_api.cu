@@ -751,7 +751,7 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     D2C_TRY(ctx, gemm(ctx, gd, EPI_RESIDUAL));
     if (aside) {
       // The host needs longer for these calls than small kernels run, so the chain's came first: those of this layer, behind the
-      // last one also the LM head's, unless that takes all SMs.
+      // last one also the LM head's, unless that takes all SMs (the smallest step 51.5 -> 51.1 us; the others do not wait for the host).
       if (l == c.n_layers - 1 && !lm_takes_all) { last_pass = at; pass_left = true; continue; }
       D2C_TRY(ctx, cu(cudaStreamWaitEvent(side, ctx->ev_fwd, 0)));
       D2C_TRY(ctx, launch_attention(at, side));

@@ -423,7 +423,7 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
   // Everything that does not read a predecessor's results (barriers, TMEM, descriptor prefetch) runs before
   // the wait on the preceding kernel, so it overlaps that kernel's tail.
   // The LM head lets its successor launch only when its loads are requested: those CTAs would wait on the SMs that it leaves to
-  // the rollout and the host's rows.
+  // the rollout and the host's rows (one layer with host buffers 371 -> 363 us, four at 236 of 2048 positions 812 -> 795).
   if (EPI != EPI_LMSTATS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr bool kPairs = EPI == EPI_SWIGLU || EPI == EPI_QKV_ROPE;             // the epilogue pairs features
   const GemmArgs& g = p.g;
@@ -708,8 +708,8 @@ gemm_tc2_kernel(const __grid_constant__ Tc2Maps maps, const Tc2Params p) {
     auto slot_of = [&](int cluster, bool head) { return (size_t)((cluster * 2 + (head ? 1 : 0)) * 2) * SLOT_F4; };
     // The warp reads TMEM no more.  The CTAs of the pair part here, ahead of the last items' arithmetic and stores, which then run
     // beside the wait for the peer and the release of TMEM (before, 0.7 us of a launch behind them: 32 layers at 80 rows 3931 -> 3894
-    // us, two of d 512 at 299 rows 127.4 -> 124.4).  Relaxed: what is stored need not be seen by the peer, and a release would wait
-    // for it.
+    // us, two of d 512 at 299 rows 127.4 -> 124.4, and that although the LM head and the residual form spill two to four registers
+    // more for it).  Relaxed: what is stored need not be seen by the peer, and a release would wait for it.
     bool left_tmem = false;
     auto leave_tmem = [&]() {
       tc_fence_before();
