@@ -16,6 +16,7 @@
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
+#include "tc2_work.cuh"
 
 namespace d2c {
 namespace {
@@ -107,28 +108,80 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32
                  "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]) : "memory");
 }
 
+// Items are numbered sequence by sequence, `mine` of them for this lane's sequence (lane l: sequence b0 + l): the lane whose items include
+// the i-th, which becomes its number among those, or -1 and i less all of them.  A warp finds it together.
+__device__ __forceinline__ int lane_of_item(int mine, int& i) {
+  int sum = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, sum, o);
+    if ((int)(threadIdx.x & 31) >= o) sum += up;
+  }
+  const unsigned behind = __ballot_sync(0xffffffffu, i < sum);
+  const int at = behind ? __ffs(behind) - 1 : 31;
+  i -= __shfl_sync(0xffffffffu, behind ? sum - mine : sum, at);
+  return behind ? at : -1;
+}
+
+// What a CTA of the forward works on: sequence, head, first row, rows (0: nothing).  By a whole warp.  A call, as its registers would
+// otherwise be taken from the softmax warps', which then spill.
+// The grid has room for all rows of all sequences, and a CTA without any still holds an SM, of whose shared memory it wants nearly all,
+// for a microsecond.  So the live ones are numbered in turn and the others come behind them; by their places in a grid of (tiles, heads,
+// sequences), where they stood between, us: 147 rows of four sequences x 1187 keys x 28 heads 33.1 -> 24.6, 260 of eight x 700 54.0 ->
+// 49.0, 300 of five x 3071 x 32 144.4 -> 133.0, 2880 of two x 4096 348.5 -> 345.5, 976 of four x 1536 and 797 x 797 no difference.  (Items
+// of two tiles first, those of one behind them: 142 where it is 134, as a head's keys then come out of the L2 no longer.)
+__device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int hq, int sm_count) {
+  const int lane = threadIdx.x & 31;
+  int i = blockIdx.x, all = 0;
+  if (batch == 1) {                                                 // (without the scan: 0.3 us of a launch)
+    const int first = row_off[0], n = row_off[1] - first, tiles = (n + AQ - 1) / AQ, width = tiles * hq > sm_count ? 2 : 1;
+    const int of = max((tiles + width - 1) >> (width - 1), 1), h = div24(i, of), r = (i - h * of) * width * AQ;
+    return make_int4(0, h, first + r, h < hq ? min(width * AQ, n - r) : 0);
+  }
+  if (batch > 32)
+    for (int b0 = 0; b0 < batch; b0 += 32)
+      all += __reduce_add_sync(0xffffffffu, b0 + lane < batch ? (row_off[b0 + lane + 1] - row_off[b0 + lane] + AQ - 1) / AQ * hq : 0);
+  for (int b0 = 0; b0 < batch; b0 += 32) {
+    const int first = b0 + lane < batch ? row_off[b0 + lane] : 0, n = b0 + lane < batch ? row_off[b0 + lane + 1] - first : 0, tiles = (n + AQ - 1) / AQ;
+    if (batch <= 32) all = __reduce_add_sync(0xffffffffu, tiles * hq);
+    const int width = all > sm_count ? 2 : 1, per = (tiles + width - 1) >> (width - 1);       // tiles of an item, items of a head
+    const int at = lane_of_item(per * hq, i);
+    if (at < 0) continue;
+    const int of = __shfl_sync(0xffffffffu, per, at), h = div24(i, of), r = (i - h * of) * width * AQ;
+    return make_int4(b0 + at, h, __shfl_sync(0xffffffffu, first, at) + r, min(width * AQ, __shfl_sync(0xffffffffu, n, at) - r));
+  }
+  return make_int4(0, 0, 0, 0);
+}
+
 template <bool kSplit>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const AttnTcParams p) {
   pdl_prologue();
   const AttnArgs& a = p.a;
-  // split: the row tile is the slowest index, so that the live ones start first (beyond them CTAs only find nothing to do)
-  const int b = kSplit ? (int)blockIdx.z % a.batch : (int)blockIdx.z, h = blockIdx.y, g = h / (a.hq / a.hkv);
   // With few selected rows every 128-row tile gets a CTA of its own (more SMs busy); otherwise a CTA
   // takes two tiles, which halves the K/V traffic per row and keeps both softmax warp groups busy.
-  const int nb = a.row_off[b + 1] - a.row_off[b];
   // With so few that SMs would idle all the same, the CTAs of a cluster share one tile's keys (p.splits of them).
-  const int splits = kSplit ? p.splits : 1, part = kSplit ? (int)blockIdx.x : 0, xtile = kSplit ? (int)blockIdx.z / a.batch : (int)blockIdx.x;
-  const bool pairs = !kSplit && ((nb + AQ - 1) / AQ) * a.hq * a.batch > p.sm_count;
-  const int r0 = a.row_off[b] + xtile * (pairs ? 2 * AQ : AQ);
-  const int nrows = min(pairs ? 2 * AQ : AQ, a.row_off[b + 1] - r0);
-  if (nrows <= 0) return;                                          // uniform in the cluster: nothing allocated yet
-  const int nq = nrows > AQ ? 2 : 1;                                // live query tiles
+  const int splits = kSplit ? p.splits : 1, part = kSplit ? (int)blockIdx.x : 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // What this CTA works on: sequence, head, first row, rows (none: nothing).  One warp works it out, and the softmax warps read it where
+  // they need it: held from here on it made them spill.
+  __shared__ int s_item[4];
+  volatile int* item = s_item;
+  if constexpr (kSplit) {
+    // The row tile is the slowest index, so that the live ones start first.  The grid has room for half of the tiles that there can be:
+    // with more rows than that every CTA takes two.  (Its other CTAs find nothing to do.)
+    const int b = (int)blockIdx.z % a.batch, r0 = a.row_off[b], nb = a.row_off[b + 1] - r0;
+    const int width = nb > (int)gridDim.z / a.batch * AQ ? 2 * AQ : AQ, at = (int)blockIdx.z / a.batch * width;
+    if (at >= nb) return;                                           // uniform in the cluster: nothing allocated yet
+    if (threadIdx.x == 0) { item[0] = b; item[1] = blockIdx.y; item[2] = r0 + at; item[3] = min(width, nb - at); }
+  } else if (warp == 0) {
+    const int4 it = forward_item(a.row_off, a.batch, a.hq, p.sm_count);
+    if (lane == 0) { item[0] = it.x; item[1] = it.y; item[2] = it.z; item[3] = it.w; }
+  }
   const int L = a.seq_len, tiles = (L + AKEYS - 1) / AKEYS;
   const int first = kSplit ? tiles * part / splits : 0, T = kSplit ? tiles * (part + 1) / splits - first : tiles;      // this CTA's key tiles (at least one)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int* status = p.status ? p.status : g_attn_status;
+  int* const status = p.status;                                     // (from the arguments at each use: held, it is two registers too many)
 
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sbase = ((uint32_t)__cvta_generic_to_shared(smem_raw) + 1023u) & ~1023u;
@@ -142,7 +195,7 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   __shared__ int abort_flag;
   const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(bars);
   auto B = [&](int i) { return bar0 + 8u * i; };
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 64) {
     for (int i = 0; i < 9; ++i) mbar_init(B(i), 1);
     mbar_init(B(9), 4); mbar_init(B(10), 4);
     mbar_init(B(11), 1); mbar_init(B(12), 1);
@@ -155,13 +208,18 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (!kSplit && item[3] <= 0) {
+    if (warp == 1) tmem_dealloc(tmem_slot, 512);
+    return;
+  }
+  const int nq = item[3] > AQ ? 2 : 1;                              // live query tiles
   const uint32_t tm = tmem_slot;                                    // tile q: S/P at q*256, O at q*256 + 128
   volatile int* abortp = &abort_flag;
-  const int kv_row0 = b * a.cache_seq + first * AKEYS;
 
   if (warp < 4) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
   if (warp == 0) {
     if (lane == 0) {
+      const int h = item[1], g = h / (a.hq / a.hkv), r0 = item[2], kv_row0 = item[0] * a.cache_seq + first * AKEYS;
       mbar_expect_tx(B(0), nq * TILE_BYTES);
       for (int q = 0; q < nq; ++q) {
         tma_load_2d(sQ(q), &tmQ, h * ADH, r0 + q * AQ, B(0));
@@ -276,7 +334,7 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     if (q < nq) {
       const int quarter = warp & 3, lrow = q * AQ + quarter * 32 + lane;
       const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-      const bool dbuf = nq == 1;                                    // one query tile: S/P alternate between the TMEM halves
+      const bool dbuf = item[3] <= AQ;                              // one query tile: S/P alternate between the TMEM halves
       const uint32_t to = tm + q * 256 + 128 + lane_base;
       const float sc = kLog2e * rsqrtf((float)ADH);
       float m_used = -INFINITY, l = 0.f;
@@ -400,8 +458,8 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       if (ok) ok = __all_sync(0xffffffffu, mbar_wait(B(11 + q), (T - 1) & 1, abortp, status, 19));
       tc_fence_after();
       if (kSplit && ok) {
-        // this CTA's share of the sum and what it is relative to, for the meeting below: over the Q tile, a row's 16-byte
-        // pieces swizzled over the banks (every MMA has read its operands)
+        // this CTA's share of the sum and what it is relative to, for the meeting below: over the Q tiles and the first K/V stage, a
+        // row's 16-byte pieces swizzled over the banks (every MMA of this query tile has read its operands; see the wait)
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
           uint32_t v[32];
@@ -412,11 +470,12 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sbase + (uint32_t)(lrow * 512 + (((c * 8 + t) ^ (lrow & 31)) << 4))),
                          "r"(v[4 * t]), "r"(v[4 * t + 1]), "r"(v[4 * t + 2]), "r"(v[4 * t + 3]) : "memory");
         }
-        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(sK(0) + (uint32_t)lrow * 8u), "f"(m_used), "f"(l) : "memory");
+        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(sK(1) + (uint32_t)lrow * 8u), "f"(m_used), "f"(l) : "memory");
       } else if (ok) {
         // Through this warp's part of its Q tile, which every MMA has read: a row's 16-byte pieces, swizzled, go in by rows and
         // come out as whole rows.  (Each thread storing its own row, 16 bytes at a time: 976 rows of four sequences x 1536 keys 107.5 us,
         // 100.7 this way, 797 x 797 20.4 and 19.9, 147 of four x 1187 28.0 and 27.5.)
+        const int h = item[1], r0 = item[2], nrows = item[3];
         const bool row_ok = lrow < nrows;
         const float inv = 1.f / l;
         const uint32_t stage = sQ(q) + (uint32_t)(quarter * 32) * 256u;
@@ -451,11 +510,12 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     cluster_sync_all();
     if (warp >= 4 && !*abortp) {
       // this CTA's share of the tile's rows, a warp a row: the parts' sums relative to the largest of their maxima
+      const int h = item[1], r0 = item[2], nrows = item[3];
       const int ra = nrows * part / splits, rb = nrows * (part + 1) / splits;
       for (int r = ra + (warp - 4); r < rb; r += 8) {
         float pm[kMaxSplits], pl[kMaxSplits], m = -INFINITY, l = 0.f;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), x[kMaxSplits];
-        const uint32_t o_at = sbase + (uint32_t)(r * 512 + ((lane ^ (r & 31)) << 4)), m_at = sK(0) + (uint32_t)r * 8u;
+        const uint32_t o_at = sbase + (uint32_t)(r * 512 + ((lane ^ (r & 31)) << 4)), m_at = sK(1) + (uint32_t)r * 8u;
 #pragma unroll
         for (int s = 0; s < kMaxSplits; ++s) {
           pm[s] = -INFINITY; pl[s] = 0.f; x[s] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -510,11 +570,11 @@ struct AbarMaps { CUtensorMap k, q[N_QBOX]; };
 struct Item { int b, key0, w, r0, nrows, bi; };      // sequence, this CTA's first key, width and rows of the tile, height of the Q box
 
 // A tile of sequence t.b's rows (the sequence's rows in tiles of almost equal width) and 256 keys; false if there is no such tile.
-__device__ __forceinline__ bool cut_item(const AttnTcParams& p, int tile, int keys, uint32_t rank, Item& t) {
-  const int first = p.a.row_off[t.b], nb = p.a.row_off[t.b + 1] - first, units = (nb + 15) >> 4;
-  const int tiles = (units * 16 + p.row_tile - 1) / p.row_tile;
+__device__ __forceinline__ bool cut_item(const AttnTcParams& p, int first, int nb, int tile, int keys, uint32_t rank, Item& t) {
+  const int units = (nb + 15) >> 4;
+  const int tiles = div24(units * 16 + p.row_tile - 1, p.row_tile);
   if (tile >= tiles) return false;
-  const int ub = units / tiles, ur = units - ub * tiles, col0 = 16 * (tile * ub + min(tile, ur));
+  const int ub = div24(units, tiles), ur = units - ub * tiles, col0 = 16 * (tile * ub + min(tile, ur));
   t.w = 16 * (ub + (tile < ur ? 1 : 0));
   t.r0 = first + col0; t.nrows = min(t.w, nb - col0);
   t.key0 = (keys * 2 + (int)rank) * AKEYS;
@@ -522,22 +582,40 @@ __device__ __forceinline__ bool cut_item(const AttnTcParams& p, int tile, int ke
   while (t.bi + 1 < N_QBOX && q_box_rows(t.bi) < (t.w >> 1)) ++t.bi;
   return true;
 }
+__device__ __forceinline__ int items_of(const AttnTcParams& p, int nb) {
+  return (p.a.seq_len + 2 * AKEYS - 1) / (2 * AKEYS) * div24(((nb + 15) & ~15) + p.row_tile - 1, p.row_tile);
+}
+// The cluster's item where the live ones are numbered in turn, so that no cluster without one stands between them.  By whole warps.
+__device__ __forceinline__ bool first_item(const AttnTcParams& p, int cluster, uint32_t rank, Item& t) {
+  const int kpairs = (p.a.seq_len + 2 * AKEYS - 1) / (2 * AKEYS);
+  int i = cluster;
+  for (int b0 = 0; b0 < p.a.batch; b0 += 32) {
+    const int b = b0 + (threadIdx.x & 31), first = b < p.a.batch ? p.a.row_off[b] : 0, nb = b < p.a.batch ? p.a.row_off[b + 1] - first : 0;
+    const int at = lane_of_item(items_of(p, nb), i);
+    t.b = b0 + at;
+    const int tile = div24(max(i, 0), kpairs);
+    if (at >= 0) return cut_item(p, __shfl_sync(0xffffffffu, first, at), __shfl_sync(0xffffffffu, nb, at), tile, i - tile * kpairs, rank, t);
+  }
+  return false;
+}
 // With `pairs` clusters that stay, each takes every pairs-th item: its n-th.
 __device__ __forceinline__ bool nth_item(const AttnTcParams& p, int n, uint32_t rank, Item& t) {
   const int kpairs = (p.a.seq_len + 2 * AKEYS - 1) / (2 * AKEYS);
   int i = (int)(blockIdx.x >> 1) + n * p.pairs;
   for (t.b = 0; t.b < p.a.batch; ++t.b) {
-    const int of = kpairs * ((((p.a.row_off[t.b + 1] - p.a.row_off[t.b] + 15) & ~15) + p.row_tile - 1) / p.row_tile);
-    if (i < of) return cut_item(p, i / kpairs, i % kpairs, rank, t);
+    const int first = p.a.row_off[t.b], nb = p.a.row_off[t.b + 1] - first, of = items_of(p, nb);
+    if (i < of) return cut_item(p, first, nb, i / kpairs, i % kpairs, rank, t);
     i -= of;
   }
   return false;
 }
 
-// kStay: a.pairs clusters do all of it, instead of one cluster an item.
-template <bool kStay>
+// How the clusters come to their items: each its own by its place in the grid, or numbered in turn, or a.pairs clusters do all of them.
+enum AbarForm { ABAR_GRID = 0, ABAR_IN_TURN = 1, ABAR_STAY = 2 };
+template <AbarForm kForm>
 __global__ void __launch_bounds__(ABAR_THREADS, 1)
 attn_abar_tc(const __grid_constant__ AbarMaps maps, const AttnTcParams p) {
+  constexpr bool kStay = kForm == ABAR_STAY;
   pdl_prologue();
   const AttnArgs& a = p.a;
   const int L = a.seq_len;
@@ -547,15 +625,19 @@ attn_abar_tc(const __grid_constant__ AbarMaps maps, const AttnTcParams p) {
   const uint16_t both = (uint16_t)(3u << (crank & ~1u));            // the pair, for multicast commits
   const int nh = a.hq / hgs, h_first = hg * nh;                     // this pair's heads (whole kv groups)
   Item it;
-  if constexpr (kStay) {
-    if (!nth_item(p, 0, rank, it)) return;                          // the whole cluster
+  // (return: the whole cluster)
+  if constexpr (kForm == ABAR_STAY) {
+    if (!nth_item(p, 0, rank, it)) return;
+  } else if constexpr (kForm == ABAR_IN_TURN) {
+    if (!first_item(p, (int)blockIdx.x >> (hgs == 4 ? 3 : hgs), rank, it)) return;
   } else {
     it.b = blockIdx.z;
-    if (!cut_item(p, blockIdx.y, (int)blockIdx.x / (2 * hgs), rank, it)) return;
+    const int first = a.row_off[it.b];
+    if (!cut_item(p, first, a.row_off[it.b + 1] - first, blockIdx.y, (int)blockIdx.x / (2 * hgs), rank, it)) return;
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int group = a.hq / a.hkv;
-  int* status = p.status ? p.status : g_attn_status;
+  int* const status = p.status;
 
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = ((uint32_t)__cvta_generic_to_shared(smem_raw) + 1023u) & ~1023u;
@@ -800,8 +882,8 @@ static int pairs_at_once(int hgs, int smem) {
     attr[0].val.clusterDim.x = 2 * hgs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int clusters = 0;
-    (void)cudaFuncSetAttribute(attn_abar_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (cudaOccupancyMaxActiveClusters(&clusters, attn_abar_tc<false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); clusters = 32 / hgs; }
+    (void)cudaFuncSetAttribute(attn_abar_tc<ABAR_GRID>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (cudaOccupancyMaxActiveClusters(&clusters, attn_abar_tc<ABAR_GRID>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); clusters = 32 / hgs; }
     n = clusters > 0 ? clusters * hgs : 1;
   }
   return n;
@@ -865,6 +947,7 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   const int smem_fwd = 6 * TILE_BYTES + 1024;
   const uint64_t kv_cols = (uint64_t)a.hkv * a.dh, kv_rows = (uint64_t)a.batch * a.cache_seq;
   const int sms = sm_count_current();
+  if (!status) D2C_CUDA_OK(cudaGetSymbolAddress(reinterpret_cast<void**>(&status), g_attn_status));
   AttnTcParams p{a, status, sms, 1, 1, 128, 0};
   const int rows_seq = expected_rows_per_seq(a);
   if (a.which != 2) {
@@ -893,7 +976,10 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
       if (s * units <= sms - 16 && key_tiles >= (s == 4 ? 16 : s + 1)) p.splits = s;
     cudaLaunchConfig_t cfg = {};
     const int xtiles = ceil_div(a.max_rows_per_seq, AQ);
-    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hq, xtiles * a.batch) : dim3(xtiles, a.hq, a.batch);
+    // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond; with shared keys clusters for half of the
+    // tiles, which take two each where that is not enough: 32 layers at 80 rows of 768 positions 3810 -> 3775 us against one for each)
+    const int most = a.hq * a.batch * ((xtiles + 1) / 2), single = a.hq * a.batch * xtiles < sms ? a.hq * a.batch * xtiles : sms;
+    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hq, (xtiles + 1) / 2 * a.batch) : dim3(most > single ? most : single);
     cfg.blockDim = dim3(FWD_THREADS); cfg.dynamicSmemBytes = smem_fwd; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -907,8 +993,8 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   if (!a.abar || a.which == 1) return D2C_OK;
   static PerDevice attr_set;
   if (attr_set.first()) {
-    D2C_CUDA_OK(cudaFuncSetAttribute(attn_abar_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAbarSmem));
-    D2C_CUDA_OK(cudaFuncSetAttribute(attn_abar_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAbarSmem));
+    for (auto* k : {attn_abar_tc<ABAR_GRID>, attn_abar_tc<ABAR_IN_TURN>, attn_abar_tc<ABAR_STAY>})
+      D2C_CUDA_OK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kAbarSmem));
   }
   const AbarCut cut = abar_cut(a);
   p.head_groups = cut.hgs; p.row_tile = cut.row_tile; p.pairs = a.pairs;
@@ -926,7 +1012,12 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     if (rc != D2C_OK) { if (a.cache[1]) a.cache[1]->forget(); return rc; }
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = p.pairs > 0 ? dim3(2 * p.pairs) : dim3(2 * p.head_groups * ceil_div(a.seq_len, 2 * AKEYS), ceil_div(a.max_rows_per_seq, p.row_tile), a.batch);
+  // Where there is room for twice as many tiles of rows as are expected, or more, the live items are numbered in turn, as in the forward:
+  // 300 rows of five sequences x 3071 keys 100.5 -> 95.8 us, 147 of four x 1187 32.4 -> 31.1, 420 of three x 1100 38.3 -> 37.8.  Finding its
+  // number takes a cluster up to 0.9 us, which it is not worth with fewer (260 of eight x 700 41.8 / 42.7) or one sequence.
+  const int xs = 2 * p.head_groups * ceil_div(a.seq_len, 2 * AKEYS), worst_tiles = ceil_div(a.max_rows_per_seq, p.row_tile);
+  const bool in_turn = a.batch > 1 && worst_tiles >= 2 * ceil_div(rows_seq, p.row_tile);
+  cfg.gridDim = p.pairs > 0 ? dim3(2 * p.pairs) : (in_turn ? dim3(xs * worst_tiles * a.batch) : dim3(xs, worst_tiles, a.batch));
   cfg.blockDim = dim3(ABAR_THREADS); cfg.dynamicSmemBytes = kAbarSmem; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -934,7 +1025,7 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
-  D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, p.pairs > 0 ? attn_abar_tc<true> : attn_abar_tc<false>, *m, p));
+  D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, p.pairs > 0 ? attn_abar_tc<ABAR_STAY> : in_turn ? attn_abar_tc<ABAR_IN_TURN> : attn_abar_tc<ABAR_GRID>, *m, p));
   count_launch(1);
   return D2C_OK;
 }
