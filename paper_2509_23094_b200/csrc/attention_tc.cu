@@ -60,7 +60,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; };
+struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, rows; };      // group: query heads of a K/V head; rows: selected rows of a query tile
 
 // ------------------------------------------------------------------------------------------------
 // Forward kernel.  One CTA owns up to 256 selected rows of one (sequence, head): two query tiles of
@@ -123,48 +123,53 @@ __device__ __forceinline__ int lane_of_item(int mine, int& i) {
   return behind ? at : -1;
 }
 
-// What a CTA of the forward works on: sequence, head, first row, rows (0: nothing).  By a whole warp.  A call, as its registers would
+// What a CTA of the forward works on: sequence, K/V head, first row, rows (0: nothing).  By a whole warp.  A call, as its registers would
 // otherwise be taken from the softmax warps', which then spill.
 // The grid has room for all rows of all sequences, and a CTA without any still holds an SM, of whose shared memory it wants nearly all,
 // for a microsecond.  So the live ones are numbered in turn and the others come behind them; by their places in a grid of (tiles, heads,
 // sequences), where they stood between, us: 147 rows of four sequences x 1187 keys x 28 heads 33.1 -> 24.6, 260 of eight x 700 54.0 ->
 // 49.0, 300 of five x 3071 x 32 144.4 -> 133.0, 2880 of two x 4096 348.5 -> 345.5, 976 of four x 1536 and 797 x 797 no difference.  (Items
 // of two tiles first, those of one behind them: 142 where it is 134, as a head's keys then come out of the L2 no longer.)
-__device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int hq, int sm_count) {
+template <bool kGroup>
+__device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int heads, int rows_, int sm_count) {
+  const int rows = kGroup ? rows_ : AQ;
   const int lane = threadIdx.x & 31;
   int i = blockIdx.x, all = 0;
+  const auto tiles_of = [&](int n) { return kGroup ? div24(n + rows - 1, rows) : (n + AQ - 1) / AQ; };
   if (batch == 1) {                                                 // (without the scan: 0.3 us of a launch)
-    const int first = row_off[0], n = row_off[1] - first, tiles = (n + AQ - 1) / AQ, width = tiles * hq > sm_count ? 2 : 1;
-    const int of = max((tiles + width - 1) >> (width - 1), 1), h = div24(i, of), r = (i - h * of) * width * AQ;
-    return make_int4(0, h, first + r, h < hq ? min(width * AQ, n - r) : 0);
+    const int first = row_off[0], n = row_off[1] - first, tiles = tiles_of(n), width = tiles * heads > sm_count ? 2 : 1;
+    const int of = max((tiles + width - 1) >> (width - 1), 1), g = div24(i, of), r = (i - g * of) * width * rows;
+    return make_int4(0, g, first + r, g < heads ? min(width * rows, n - r) : 0);
   }
   if (batch > 32)
     for (int b0 = 0; b0 < batch; b0 += 32)
-      all += __reduce_add_sync(0xffffffffu, b0 + lane < batch ? (row_off[b0 + lane + 1] - row_off[b0 + lane] + AQ - 1) / AQ * hq : 0);
+      all += __reduce_add_sync(0xffffffffu, b0 + lane < batch ? tiles_of(row_off[b0 + lane + 1] - row_off[b0 + lane]) * heads : 0);
   for (int b0 = 0; b0 < batch; b0 += 32) {
-    const int first = b0 + lane < batch ? row_off[b0 + lane] : 0, n = b0 + lane < batch ? row_off[b0 + lane + 1] - first : 0, tiles = (n + AQ - 1) / AQ;
-    if (batch <= 32) all = __reduce_add_sync(0xffffffffu, tiles * hq);
+    const int first = b0 + lane < batch ? row_off[b0 + lane] : 0, n = b0 + lane < batch ? row_off[b0 + lane + 1] - first : 0, tiles = tiles_of(n);
+    if (batch <= 32) all = __reduce_add_sync(0xffffffffu, tiles * heads);
     const int width = all > sm_count ? 2 : 1, per = (tiles + width - 1) >> (width - 1);       // tiles of an item, items of a head
-    const int at = lane_of_item(per * hq, i);
+    const int at = lane_of_item(per * heads, i);
     if (at < 0) continue;
-    const int of = __shfl_sync(0xffffffffu, per, at), h = div24(i, of), r = (i - h * of) * width * AQ;
-    return make_int4(b0 + at, h, __shfl_sync(0xffffffffu, first, at) + r, min(width * AQ, __shfl_sync(0xffffffffu, n, at) - r));
+    const int of = __shfl_sync(0xffffffffu, per, at), g = div24(i, of), r = (i - g * of) * width * rows;
+    return make_int4(b0 + at, g, __shfl_sync(0xffffffffu, first, at) + r, min(width * rows, __shfl_sync(0xffffffffu, n, at) - r));
   }
   return make_int4(0, 0, 0, 0);
 }
 
-template <bool kSplit>
+// kGroup: a K/V head has several query heads (one: the tile's divisions by their number fold away, 0.3 us of a CTA).
+template <bool kSplit, bool kGroup>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const AttnTcParams p) {
   pdl_prologue();
   const AttnArgs& a = p.a;
+  const int group = kGroup ? p.group : 1, tile_rows = kGroup ? p.rows : AQ;
   // With few selected rows every 128-row tile gets a CTA of its own (more SMs busy); otherwise a CTA
   // takes two tiles, which halves the K/V traffic per row and keeps both softmax warp groups busy.
   // With so few that SMs would idle all the same, the CTAs of a cluster share one tile's keys (p.splits of them).
   const int splits = kSplit ? p.splits : 1, part = kSplit ? (int)blockIdx.x : 0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // What this CTA works on: sequence, head, first row, rows (none: nothing).  One warp works it out, and the softmax warps read it where
+  // What this CTA works on: sequence, K/V head, first row, rows (none: nothing).  One warp works it out, and the softmax warps read it where
   // they need it: held from here on it made them spill.
   __shared__ int s_item[4];
   volatile int* item = s_item;
@@ -172,11 +177,11 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     // The row tile is the slowest index, so that the live ones start first.  The grid has room for half of the tiles that there can be:
     // with more rows than that every CTA takes two.  (Its other CTAs find nothing to do.)
     const int b = (int)blockIdx.z % a.batch, r0 = a.row_off[b], nb = a.row_off[b + 1] - r0;
-    const int width = nb > (int)gridDim.z / a.batch * AQ ? 2 * AQ : AQ, at = (int)blockIdx.z / a.batch * width;
+    const int width = nb > (int)gridDim.z / a.batch * tile_rows ? 2 * tile_rows : tile_rows, at = (int)blockIdx.z / a.batch * width;
     if (at >= nb) return;                                           // uniform in the cluster: nothing allocated yet
     if (threadIdx.x == 0) { item[0] = b; item[1] = blockIdx.y; item[2] = r0 + at; item[3] = min(width, nb - at); }
   } else if (warp == 0) {
-    const int4 it = forward_item(a.row_off, a.batch, a.hq, p.sm_count);
+    const int4 it = forward_item<kGroup>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count);
     if (lane == 0) { item[0] = it.x; item[1] = it.y; item[2] = it.z; item[3] = it.w; }
   }
   const int L = a.seq_len, tiles = (L + AKEYS - 1) / AKEYS;
@@ -212,18 +217,18 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     if (warp == 1) tmem_dealloc(tmem_slot, 512);
     return;
   }
-  const int nq = item[3] > AQ ? 2 : 1;                              // live query tiles
+  const int nq = item[3] > tile_rows ? 2 : 1;                          // live query tiles
   const uint32_t tm = tmem_slot;                                    // tile q: S/P at q*256, O at q*256 + 128
   volatile int* abortp = &abort_flag;
 
   if (warp < 4) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
   if (warp == 0) {
     if (lane == 0) {
-      const int h = item[1], g = h / (a.hq / a.hkv), r0 = item[2], kv_row0 = item[0] * a.cache_seq + first * AKEYS;
-      mbar_expect_tx(B(0), nq * TILE_BYTES);
+      const int g = item[1], r0 = item[2], kv_row0 = item[0] * a.cache_seq + first * AKEYS;
+      mbar_expect_tx(B(0), nq * tile_rows * group * ADH * 2);
       for (int q = 0; q < nq; ++q) {
-        tma_load_2d(sQ(q), &tmQ, h * ADH, r0 + q * AQ, B(0));
-        tma_load_2d(sQ(q) + HALF_BYTES, &tmQ, h * ADH + 64, r0 + q * AQ, B(0));
+        tma_load_3d(sQ(q), &tmQ, 0, g * group, r0 + q * tile_rows, B(0));
+        tma_load_3d(sQ(q) + HALF_BYTES, &tmQ, 64, g * group, r0 + q * tile_rows, B(0));
       }
       int issued = 0;
       for (int j = 0; j < T; ++j) {
@@ -334,7 +339,7 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     if (q < nq) {
       const int quarter = warp & 3, lrow = q * AQ + quarter * 32 + lane;
       const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-      const bool dbuf = item[3] <= AQ;                              // one query tile: S/P alternate between the TMEM halves
+      const bool dbuf = item[3] <= tile_rows;                            // one query tile: S/P alternate between the TMEM halves
       const uint32_t to = tm + q * 256 + 128 + lane_base;
       const float sc = kLog2e * rsqrtf((float)ADH);
       float m_used = -INFINITY, l = 0.f;
@@ -475,8 +480,9 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         // Through this warp's part of its Q tile, which every MMA has read: a row's 16-byte pieces, swizzled, go in by rows and
         // come out as whole rows.  (Each thread storing its own row, 16 bytes at a time: 976 rows of four sequences x 1536 keys 107.5 us,
         // 100.7 this way, 797 x 797 20.4 and 19.9, 147 of four x 1187 28.0 and 27.5.)
-        const int h = item[1], r0 = item[2], nrows = item[3];
-        const bool row_ok = lrow < nrows;
+        // A tile's row is (selected row, head of the group), the head the faster: its outputs lie one behind the other too.
+        const int live = min(item[3] - q * tile_rows, tile_rows) * group, m0 = quarter * 32;
+        const size_t first_out = (size_t)(item[2] + q * tile_rows) * a.hq + item[1] * group;
         const float inv = 1.f / l;
         const uint32_t stage = sQ(q) + (uint32_t)(quarter * 32) * 256u;
 #pragma unroll 1
@@ -493,15 +499,20 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                          "r"(pack_bf16(__uint_as_float(v[8 * t + 6]) * inv, __uint_as_float(v[8 * t + 7]) * inv)) : "memory");
         }
         __syncwarp();
+        int sel = kGroup ? div24(m0 + (lane >> 4), group) : m0 + (lane >> 4), head = m0 + (lane >> 4) - sel * group;
+        const int step = 2 / min(group, 4), rest = group > 2 ? 2 : 0;      // two of the tile's rows on, in selected rows and heads
 #pragma unroll 4
         for (int i = 0; i < 16; ++i) {
-          const int r = 2 * i + (lane >> 4), pc = lane & 15, row = lrow - lane + r;
+          const int r = 2 * i + (lane >> 4), pc = lane & 15;
           uint4 w;
           asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w)
                        : "r"(stage + (uint32_t)(r * 256 + ((pc ^ (r & 15)) << 4))) : "memory");
-          if (row < nrows) reinterpret_cast<uint4*>(a.o + (size_t)(r0 + row) * ((size_t)a.hq * ADH) + (size_t)h * ADH)[pc] = w;
+          if (m0 + r < live) reinterpret_cast<uint4*>(a.o + (first_out + (size_t)sel * a.hq + head) * ADH)[pc] = w;
+          sel += step; head += rest;
+          if (kGroup && head >= group) { head -= group; ++sel; }
         }
-        if (row_ok) a.lse[(size_t)(r0 + lrow) * a.hq + h] = (m_used + log2f(l)) * kLn2;
+        sel = kGroup ? div24(m0 + lane, group) : m0 + lane;
+        if (m0 + lane < live) a.lse[first_out + (size_t)sel * a.hq + (m0 + lane - sel * group)] = (m_used + log2f(l)) * kLn2;
       }
     }
   }
@@ -510,9 +521,11 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     cluster_sync_all();
     if (warp >= 4 && !*abortp) {
       // this CTA's share of the tile's rows, a warp a row: the parts' sums relative to the largest of their maxima
-      const int h = item[1], r0 = item[2], nrows = item[3];
-      const int ra = nrows * part / splits, rb = nrows * (part + 1) / splits;
-      for (int r = ra + (warp - 4); r < rb; r += 8) {
+      const int first_live = min(item[3], tile_rows) * group, live = first_live + (item[3] > tile_rows ? (item[3] - tile_rows) * group : 0);
+      const int ra = live * part / splits, rb = live * (part + 1) / splits;
+      for (int n = ra + (warp - 4); n < rb; n += 8) {
+        const int q = n >= first_live ? 1 : 0, mine = n - q * first_live, r = q * AQ + mine, sel = kGroup ? div24(mine, group) : mine;
+        const size_t at = (size_t)(item[2] + q * tile_rows + sel) * a.hq + item[1] * group + mine - sel * group;
         float pm[kMaxSplits], pl[kMaxSplits], m = -INFINITY, l = 0.f;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), x[kMaxSplits];
         const uint32_t o_at = sbase + (uint32_t)(r * 512 + ((lane ^ (r & 31)) << 4)), m_at = sK(1) + (uint32_t)r * 8u;
@@ -536,9 +549,8 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
           acc.x = fmaf(x[s].x, w, acc.x); acc.y = fmaf(x[s].y, w, acc.y); acc.z = fmaf(x[s].z, w, acc.z); acc.w = fmaf(x[s].w, w, acc.w);
         }
         const float inv = 1.f / l;
-        bf16* dst = a.o + (size_t)(r0 + r) * ((size_t)a.hq * ADH) + (size_t)h * ADH;
-        reinterpret_cast<uint2*>(dst)[lane] = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
-        if (lane == 0) a.lse[(size_t)(r0 + r) * a.hq + h] = (m + log2f(l)) * kLn2;
+        reinterpret_cast<uint2*>(a.o + at * ADH)[lane] = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+        if (lane == 0) a.lse[at] = (m + log2f(l)) * kLn2;
       }
     }
     __syncwarp();
@@ -862,7 +874,7 @@ attn_abar_tc(const __grid_constant__ AbarMaps maps, const AttnTcParams p) {
 
 // True if the tcgen05 kernels can take this problem (otherwise the caller uses the mma.sync ones).
 bool attention_tc_supported(const AttnArgs& a) {
-  return a.dh == ADH && a.hq <= 512 && a.q_rows >= AQ && (long long)a.batch * a.cache_seq >= AKEYS && (a.ldq & 7) == 0 &&
+  return a.dh == ADH && a.hq <= 512 && a.hq / a.hkv <= AQ && a.q_rows >= AQ && (long long)a.batch * a.cache_seq >= AKEYS && (a.ldq & 7) == 0 &&
          (reinterpret_cast<uintptr_t>(a.q) & 15) == 0 && (reinterpret_cast<uintptr_t>(a.kc) & 15) == 0 &&
          (reinterpret_cast<uintptr_t>(a.vc) & 15) == 0;
 }
@@ -948,13 +960,17 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   const uint64_t kv_cols = (uint64_t)a.hkv * a.dh, kv_rows = (uint64_t)a.batch * a.cache_seq;
   const int sms = sm_count_current();
   if (!status) D2C_CUDA_OK(cudaGetSymbolAddress(reinterpret_cast<void**>(&status), g_attn_status));
-  AttnTcParams p{a, status, sms, 1, 1, 128, 0};
+  // A query tile holds the rows of all query heads of a K/V head, (row, head) by (row, head), as many whole rows as there is room for: 18
+  // rows of seven heads, where a head's own rows filled their last tile only in part.  Forward alone, a head's rows / a group's, us, 28 heads
+  // over 4: 260 rows of eight sequences x 700 keys 48.6 / 33.6, 147 of four x 1187 24.5 / 21.2, 976 of four x 1536 100.4 / 93.6.
+  const int group = a.hq / a.hkv, tile_rows = AQ / group;
+  AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, tile_rows};
   const int rows_seq = expected_rows_per_seq(a);
   if (a.which != 2) {
     static PerDevice attr_set;
     if (attr_set.first()) {
-      D2C_CUDA_OK(cudaFuncSetAttribute(attn_fwd_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_fwd));
-      D2C_CUDA_OK(cudaFuncSetAttribute(attn_fwd_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_fwd));
+      for (auto* k : {attn_fwd_tc<false, false>, attn_fwd_tc<false, true>, attn_fwd_tc<true, false>, attn_fwd_tc<true, true>})
+        D2C_CUDA_OK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_fwd));
     }
     struct Maps { CUtensorMap q, k, v; } fresh, *m = &fresh;
     bool made = false;
@@ -963,7 +979,7 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
       made = a.cache[0]->same(a.q, a.kc, a.vc, a.q_rows, a.hq, a.ldq, (long long)kv_rows, (long long)kv_cols, 3);
     }
     if (!made) {
-      int rc = make_bf16_map(&m->q, a.q, (uint64_t)a.q_rows, (uint64_t)a.hq * a.dh, (uint64_t)a.ldq, 128);
+      int rc = make_bf16_head_map(&m->q, a.q, (uint64_t)a.q_rows, (uint64_t)a.hq, (uint64_t)a.ldq, (uint32_t)tile_rows, (uint32_t)group);
       if (rc == D2C_OK) rc = make_bf16_map(&m->k, a.kc, kv_rows, kv_cols, kv_cols, 128);
       if (rc == D2C_OK) rc = make_bf16_map(&m->v, a.vc, kv_rows, kv_cols, kv_cols, 128);
       if (rc != D2C_OK) { if (a.cache[0]) a.cache[0]->forget(); return rc; }
@@ -971,15 +987,15 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     // Few tiles of 128 rows (expected): 2 to 4 CTAs share a tile's keys while all of them still run at once.  Four only
     // for many key tiles: measured alone at 32 heads (us, 1 / 2 / 3 / 4 CTAs) 768 keys 20.4 / 18.4 / 16.4 / 17.3,
     // 2048 keys 36.8 / 27.6 / 24.6 / 22.5, 4096 keys 64.4 / 43.0 / 36.8 / 31.7.
-    const int units = ceil_div(rows_seq, AQ) * a.hq * a.batch, key_tiles = ceil_div(a.seq_len, AKEYS);
+    const int units = ceil_div(rows_seq, tile_rows) * a.hkv * a.batch, key_tiles = ceil_div(a.seq_len, AKEYS);
     for (int s = 2; s <= kMaxSplits; ++s)
       if (s * units <= sms - 16 && key_tiles >= (s == 4 ? 16 : s + 1)) p.splits = s;
     cudaLaunchConfig_t cfg = {};
-    const int xtiles = ceil_div(a.max_rows_per_seq, AQ);
+    const int xtiles = ceil_div(a.max_rows_per_seq, tile_rows);
     // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond; with shared keys clusters for half of the
     // tiles, which take two each where that is not enough: 32 layers at 80 rows of 768 positions 3810 -> 3775 us against one for each)
-    const int most = a.hq * a.batch * ((xtiles + 1) / 2), single = a.hq * a.batch * xtiles < sms ? a.hq * a.batch * xtiles : sms;
-    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hq, (xtiles + 1) / 2 * a.batch) : dim3(most > single ? most : single);
+    const int most = a.hkv * a.batch * ((xtiles + 1) / 2), single = a.hkv * a.batch * xtiles < sms ? a.hkv * a.batch * xtiles : sms;
+    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hkv, (xtiles + 1) / 2 * a.batch) : dim3(most > single ? most : single);
     cfg.blockDim = dim3(FWD_THREADS); cfg.dynamicSmemBytes = smem_fwd; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -987,7 +1003,8 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = p.splits; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = p.splits > 1 ? 2 : 1;
-    D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, p.splits > 1 ? attn_fwd_tc<true> : attn_fwd_tc<false>, m->q, m->k, m->v, p));
+    auto* kernel = p.splits > 1 ? (group > 1 ? attn_fwd_tc<true, true> : attn_fwd_tc<true, false>) : (group > 1 ? attn_fwd_tc<false, true> : attn_fwd_tc<false, false>);
+    D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, m->q, m->k, m->v, p));
     count_launch(1);
   }
   if (!a.abar || a.which == 1) return D2C_OK;
