@@ -60,7 +60,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, rows; };      // group: query heads of a K/V head; rows: selected rows of a query tile
+struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, rows, split_last; };      // group: query heads of a K/V head; rows: selected rows of a query tile
 
 // ------------------------------------------------------------------------------------------------
 // Forward kernel.  One CTA owns up to 256 selected rows of one (sequence, head): two query tiles of
@@ -130,28 +130,48 @@ __device__ __forceinline__ int lane_of_item(int mine, int& i) {
 // sequences), where they stood between, us: 147 rows of four sequences x 1187 keys x 28 heads 33.1 -> 24.6, 260 of eight x 700 54.0 ->
 // 49.0, 300 of five x 3071 x 32 144.4 -> 133.0, 2880 of two x 4096 348.5 -> 345.5, 976 of four x 1536 and 797 x 797 no difference.  (Items
 // of two tiles first, those of one behind them: 142 where it is 134, as a head's keys then come out of the L2 no longer.)
-template <bool kGroup>
+template <bool kGroup, bool kSplitLast>
 __device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int heads, int rows_, int sm_count) {
   const int rows = kGroup ? rows_ : AQ;
   const int lane = threadIdx.x & 31;
-  int i = blockIdx.x, all = 0;
+  int i = blockIdx.x, all = 0, pairs = 0, half = -1;                // tiles, and pairs of them
   const auto tiles_of = [&](int n) { return kGroup ? div24(n + rows - 1, rows) : (n + AQ - 1) / AQ; };
+  // What is left over behind whole waves of pairs, where it is so little that its tiles can have an SM each, is split into tiles: a pair
+  // takes 1.6 times as long as a tile.  Forward alone, us: 976 rows of four sequences x 1536 keys x 28 heads over 4 (448 pairs) 93.6 -> 88.0,
+  // 420 of three x 1100 x 32 42.5 -> 39.3, 300 of five x 3071 133.0 -> 129.9.
+  const auto split_last = [&]() {
+    const int whole = div24(pairs, sm_count) * sm_count;
+    if (all > sm_count && 2 * (pairs - whole) <= sm_count && i >= whole) { half = (i - whole) & 1; i = whole + ((i - whole) >> 1); }
+  };
+  const auto item_of = [&](int b, int g, int first, int n, int r, int width) {
+    if (kSplitLast && half >= 0) { r += half * rows; width = 1; }
+    return make_int4(b, g, first + r, min(width * rows, n - r));
+  };
   if (batch == 1) {                                                 // (without the scan: 0.3 us of a launch)
     const int first = row_off[0], n = row_off[1] - first, tiles = tiles_of(n), width = tiles * heads > sm_count ? 2 : 1;
-    const int of = max((tiles + width - 1) >> (width - 1), 1), g = div24(i, of), r = (i - g * of) * width * rows;
-    return make_int4(0, g, first + r, g < heads ? min(width * rows, n - r) : 0);
+    all = tiles * heads; pairs = ((tiles + 1) >> 1) * heads;
+    if (kSplitLast) split_last();
+    const int of = max((tiles + width - 1) >> (width - 1), 1), g = div24(i, of);
+    return g < heads ? item_of(0, g, first, n, (i - g * of) * width * rows, width) : make_int4(0, 0, 0, 0);
   }
-  if (batch > 32)
-    for (int b0 = 0; b0 < batch; b0 += 32)
-      all += __reduce_add_sync(0xffffffffu, b0 + lane < batch ? tiles_of(row_off[b0 + lane + 1] - row_off[b0 + lane]) * heads : 0);
-  for (int b0 = 0; b0 < batch; b0 += 32) {
-    const int first = b0 + lane < batch ? row_off[b0 + lane] : 0, n = b0 + lane < batch ? row_off[b0 + lane + 1] - first : 0, tiles = tiles_of(n);
-    if (batch <= 32) all = __reduce_add_sync(0xffffffffu, tiles * heads);
-    const int width = all > sm_count ? 2 : 1, per = (tiles + width - 1) >> (width - 1);       // tiles of an item, items of a head
-    const int at = lane_of_item(per * heads, i);
+  int first = 0, n = 0, tiles = 0;
+  const auto load = [&](int b0) {
+    first = b0 + lane < batch ? row_off[b0 + lane] : 0; n = b0 + lane < batch ? row_off[b0 + lane + 1] - first : 0; tiles = tiles_of(n);
+  };
+  const int last = (batch - 1) & ~31;                               // (up to 32 sequences are loaded once)
+  for (int b0 = 0; b0 <= last; b0 += 32) {
+    load(b0);
+    all += __reduce_add_sync(0xffffffffu, tiles * heads);
+    if (kSplitLast) pairs += __reduce_add_sync(0xffffffffu, ((tiles + 1) >> 1) * heads);
+  }
+  const int width = all > sm_count ? 2 : 1;                         // tiles of an item
+  if (kSplitLast) split_last();
+  for (int b0 = 0; b0 <= last; b0 += 32) {
+    if (last > 0) load(b0);
+    const int per = (tiles + width - 1) >> (width - 1), at = lane_of_item(per * heads, i);      // per: items of a head
     if (at < 0) continue;
-    const int of = __shfl_sync(0xffffffffu, per, at), g = div24(i, of), r = (i - g * of) * width * rows;
-    return make_int4(b0 + at, g, __shfl_sync(0xffffffffu, first, at) + r, min(width * rows, __shfl_sync(0xffffffffu, n, at) - r));
+    const int of = __shfl_sync(0xffffffffu, per, at), g = div24(i, of);
+    return item_of(b0 + at, g, __shfl_sync(0xffffffffu, first, at), __shfl_sync(0xffffffffu, n, at), (i - g * of) * width * rows, width);
   }
   return make_int4(0, 0, 0, 0);
 }
@@ -181,7 +201,8 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     if (at >= nb) return;                                           // uniform in the cluster: nothing allocated yet
     if (threadIdx.x == 0) { item[0] = b; item[1] = blockIdx.y; item[2] = r0 + at; item[3] = min(width, nb - at); }
   } else if (warp == 0) {
-    const int4 it = forward_item<kGroup>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count);
+    const int4 it = p.split_last ? forward_item<kGroup, true>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count)
+                                 : forward_item<kGroup, false>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count);
     if (lane == 0) { item[0] = it.x; item[1] = it.y; item[2] = it.z; item[3] = it.w; }
   }
   const int L = a.seq_len, tiles = (L + AKEYS - 1) / AKEYS;
@@ -964,7 +985,7 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   // rows of seven heads, where a head's own rows filled their last tile only in part.  Forward alone, a head's rows / a group's, us, 28 heads
   // over 4: 260 rows of eight sequences x 700 keys 48.6 / 33.6, 147 of four x 1187 24.5 / 21.2, 976 of four x 1536 100.4 / 93.6.
   const int group = a.hq / a.hkv, tile_rows = AQ / group;
-  AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, tile_rows};
+  AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, tile_rows, 0};
   const int rows_seq = expected_rows_per_seq(a);
   if (a.which != 2) {
     static PerDevice attr_set;
@@ -995,7 +1016,9 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond; with shared keys clusters for half of the
     // tiles, which take two each where that is not enough: 32 layers at 80 rows of 768 positions 3810 -> 3775 us against one for each)
     const int most = a.hkv * a.batch * ((xtiles + 1) / 2), single = a.hkv * a.batch * xtiles < sms ? a.hkv * a.batch * xtiles : sms;
-    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hkv, (xtiles + 1) / 2 * a.batch) : dim3(most > single ? most : single);
+    const int pairs = ceil_div(ceil_div(rows_seq, tile_rows), 2) * a.hkv * a.batch;      // (expected; where none are to be split, looking for them costs 0.4 us)
+    p.split_last = units > sms && pairs > sms && pairs % sms > 0 && 2 * (pairs % sms) <= sms;
+    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hkv, (xtiles + 1) / 2 * a.batch) : dim3((most > single ? most : single) + (p.split_last ? sms / 2 : 0));
     cfg.blockDim = dim3(FWD_THREADS); cfg.dynamicSmemBytes = smem_fwd; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
