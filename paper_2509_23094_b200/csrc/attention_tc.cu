@@ -927,27 +927,37 @@ static int expected_rows_per_seq(const AttnArgs& a) {
   return ceil_div(rows > 0 ? rows : 1, a.batch);
 }
 
-struct AbarCut { int hgs, row_tile, ctas; };
+struct AbarCut { int hgs, row_tile, ctas, waves; };
 static AbarCut abar_cut(const AttnArgs& a, float* us = nullptr) {
   // How the work is cut: row tiles of 64, 128 or 256 rows, heads shared by 1, 2 or 4 pairs (whole kv groups each); the
   // cheapest by this estimate of waves x time of a CTA (us, measured: a head of a 256-row tile takes 1.8, of a narrow one
   // the loads' 0.5; 6 for set-up, first loads and output; 2 for the meeting).  The row count is an expectation (worst case
   // if there is none): it decides how the work is cut, not what is covered.  Beside other kernels the fewest SMs are best.
   const int kpairs = ceil_div(a.seq_len, 2 * AKEYS), kv_group = a.hq / a.hkv;
-  const int rows_seq = expected_rows_per_seq(a);
+  const int rows_seq = expected_rows_per_seq(a), units = ceil_div(rows_seq, 16);
   float best = 1e30f;
-  AbarCut cut = {1, 16, 2 * kpairs * a.batch * ceil_div(rows_seq, 16)};       // (more than 128 heads)
-  for (int hgs = 1; hgs <= (a.beside || a.pairs > 0 ? 1 : 4); hgs *= 2) {
-    if (a.hq % hgs || (a.hq / hgs) % kv_group) continue;
-    for (int tile = 256; tile >= 64; tile /= 2) {
-      const int nh = a.hq / hgs, tiles = ceil_div(rows_seq, tile), w = 16 * ceil_div(ceil_div(rows_seq, 16), tiles);
-      if (tile * nh > ABAR_MAX_ROWS * 32) continue;                 // the staged log-sum-exp
-      const int at_once = a.pairs > 0 ? a.pairs : pairs_at_once(hgs, kAbarSmem);
-      const float per_head = 0.3f + 1.5f * (float)w / 256.f;
-      const float est = (float)ceil_div(kpairs * a.batch * tiles * hgs, at_once) * ((float)nh * (per_head > 0.5f ? per_head : 0.5f) + 6.f + (hgs > 1 ? 2.f : 0.f));
-      if (est < best) { best = est; cut = {hgs, tile, 2 * kpairs * a.batch * tiles * hgs}; }
-    }
-  }
+  AbarCut cut = {1, 16, 2 * kpairs * a.batch * units, 1};         // (more than 128 heads)
+  auto consider = [&](int hgs, int tiles, int tile) {
+    const int nh = a.hq / hgs, w = 16 * ceil_div(units, tiles);
+    if (tile * nh > ABAR_MAX_ROWS * 32) return;                     // the staged log-sum-exp
+    const int at_once = a.pairs > 0 ? a.pairs : pairs_at_once(hgs, kAbarSmem), waves = ceil_div(kpairs * a.batch * tiles * hgs, at_once);
+    const float per_head = 0.3f + 1.5f * (float)w / 256.f;
+    const float est = (float)waves * ((float)nh * (per_head > 0.5f ? per_head : 0.5f) + 6.f + (hgs > 1 ? 2.f : 0.f));
+    if (est < best) { best = est; cut = {hgs, tile, 2 * kpairs * a.batch * tiles * hgs, waves}; }
+  };
+  const int most_hgs = a.beside || a.pairs > 0 ? 1 : 4;
+  auto shared = [&](int hgs) { return a.hq % hgs == 0 && (a.hq / hgs) % kv_group == 0; };
+  for (int hgs = 1; hgs <= most_hgs; hgs *= 2)
+    for (int tile = 256; tile >= 64 && shared(hgs); tile /= 2) consider(hgs, ceil_div(rows_seq, tile), tile);
+  // Where that takes several waves, any number of tiles between: 976 rows of four sequences x 1536 keys took three waves of half of 28
+  // heads each, and six tiles of 176 rows take two (four layers 5823 -> 5793 us; 1012 rows x 1500, 32 heads, three layers 1342 -> 1338).  A
+  // tile has room for sixteen rows a sequence more than are expected, so that a few more do not make another tile.
+  if (cut.waves > 1 && a.pairs == 0 && !a.beside)
+    for (int hgs = 1; hgs <= most_hgs; hgs *= 2)
+      for (int tiles = ceil_div(units, 16); tiles <= ceil_div(units, 4) && shared(hgs); ++tiles) {
+        const int tile = 16 * ceil_div(units + 1, tiles);
+        consider(hgs, tiles, tile < ABAR_MAX_ROWS ? tile : ABAR_MAX_ROWS);
+      }
   if (us) *us = best;
   return cut;
 }
