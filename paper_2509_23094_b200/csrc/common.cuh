@@ -223,6 +223,29 @@ int launch_rollout(const RolloutArgs& a, cudaStream_t st);
 static const int kRolloutSplit = 16;
 static const int kRolloutCluster = 8;          // CTAs (SMs) per sequence of the single launch
 
+// ---- a small model's step in one launch (small_step.cu) ------------------------------------------
+constexpr int kSmallCluster = 16, kSmallMaxTiles = 64, kSmallMaxBatch = 16, kSmallMaxLayers = 8, kSmallMaxClusters = 16, kSmallSmem = 196 * 1024;
+struct SmallLayer { const bf16 *wqkv, *bqkv, *wo, *w_gate, *w_up, *w_down, *g_attn, *g_ffn; };
+struct SmallArgs {
+  SelectArgs sel;
+  SmallLayer layer[kSmallMaxLayers]; const bf16 *g_final, *w_lm;
+  const bf16* h0; bf16* x; bf16* layer_in; float* logits;        // layer_in, logits: optional outputs
+  bool h0_far;                                                   // h0 lies in host memory
+  int n_layers, d, hq, hkv, ffn, vocab, cache_seq, depth; float eps;
+  size_t rows_cap;                                               // rows of a layer in layer_in
+  const float2* rope; bf16 *kc, *vc; size_t cache_layer;
+  bf16 *q, *o, *hmid; float* lse; float* abar; size_t abar_layer;
+  float *c, *conf; int32_t* pred; CopyOut copies;
+  int32_t* clear; int n_clear;                                   // words set to 0 on the way
+  int2* n_word; int n_tag;                                       // optional host words: the row count, and which step wrote it
+  uint32_t* sync; int32_t* status;                               // two counters that are zero between launches
+  float4* lm_stats; float* rp;   // scratch, see small_step_scratch
+};
+int small_step_clusters();                                       // clusters that fit the GPU together (0: none)
+// Places the scratch of a launch from `base` on (null out: only its size); floats.
+size_t small_step_scratch(const SmallArgs& a, int clusters, float* base, SmallArgs* out);
+int launch_small_step(const SmallArgs& a, int clusters, cudaStream_t st);
+
 }  // namespace d2c
 
 namespace d2c {

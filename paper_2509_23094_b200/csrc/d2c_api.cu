@@ -100,7 +100,7 @@ static size_t carve(const d2c_config& c, void* base, Buffers* out) {
   b.kcache = w.take<bf16>((size_t)c.n_layers * R * kv);
   b.vcache = w.take<bf16>((size_t)c.n_layers * R * kv);
   b.conf = w.take<float>(R); b.c = w.take<float>(R); b.key = w.take<float>(R);
-  b.pred = w.take<int32_t>(R); b.status = w.take<int32_t>(4);
+  b.pred = w.take<int32_t>(R); b.status = w.take<int32_t>(64);                 // (four status words; counters of the one-launch step from the 32nd on)
   b.sel_idx = w.take<int32_t>(R); b.row_seq = w.take<int32_t>(R); b.row_off = w.take<int32_t>(B + 1);
   b.lm_rows = w.take<int32_t>(R); b.lm_off = w.take<int32_t>(B + 1); b.slot_of_pos = w.take<int32_t>(R);
   b.rank_s = w.take<int32_t>(R); b.rank_lm = w.take<int32_t>(R); b.n_b = w.take<int32_t>(B); b.nm_b = w.take<int32_t>(B);
@@ -160,12 +160,15 @@ struct d2c_ctx {
   int32_t* hint_dev[2] = {nullptr, nullptr};
   cudaEvent_t ev_hint[2] = {nullptr, nullptr};
   long long hint_step[2] = {-1, -1};     // step number whose count the word holds
+  bool hint_tagged[2] = {false, false};  // it was a step in one launch: it writes its number behind the count, in one store
   long long step_no = 0;
   bool few_rows = false;                 // this step's regime: at most 128 rows expected
   std::vector<MapCache> maps;            // six launches of each layer (QKV, forward, probabilities, output, gate/up, down), LM head
   int max_pairs = 0;                     // SM pairs the projections of this step may use (0: all)
   int narrow_pairs = 0;                  // those 64-token tiles may spread over (0: all)
   int lm_pairs = 0;                      // those the LM head may use (0: all)
+  int small_clusters = 0;                // clusters of the kernel that does the whole step (0: the model is not one for it)
+  bool host_call = false, h0_far = false;      // in d2c_step_host; its h0 lies in host memory
   WorkPlan plan{};                       // the pair kernel's launches of the current step
   int pair_launches = 0;                 // how many of them are enqueued
   int used_batch = 0, used_seq = 0;      // the (batch, seq_len) of the first step: the per-position state is laid out for it
@@ -303,6 +306,41 @@ static void* mapped(const void* p, size_t bytes) {
 }
 #define D2C_TRY(ctx, expr) do { int rc__ = (expr); if (rc__ != D2C_OK) return pass((ctx), rc__); } while (0)
 
+// The arguments of a step in one launch, but for those of the call.
+static SmallArgs small_args(const d2c_ctx* ctx, int batch, int seq_len) {
+  const d2c_config& c = ctx->cfg;
+  const Buffers& b = ctx->buf;
+  SmallArgs a{};
+  a.sel.batch = batch; a.sel.seq_len = seq_len;
+  for (int l = 0; l < c.n_layers; ++l)
+    a.layer[l] = SmallLayer{ctx->wqkv[l], ctx->bqkv[l], ctx->wo[l], ctx->w_gate[l], ctx->w_up[l], ctx->w_down[l], ctx->g_attn[l], ctx->g_ffn[l]};
+  a.g_final = ctx->g_final; a.w_lm = ctx->w_lm;
+  a.n_layers = c.n_layers; a.d = c.d_model; a.hq = c.n_q_heads; a.hkv = c.n_kv_heads; a.ffn = c.d_ffn; a.vocab = c.vocab;
+  a.cache_seq = c.max_seq; a.depth = rollout_depth(c); a.eps = c.rms_eps;
+  a.rope = b.rope; a.kc = b.kcache; a.vc = b.vcache; a.cache_layer = (size_t)c.max_batch * c.max_seq * c.n_kv_heads * c.head_dim;
+  a.q = b.qkv; a.o = b.o; a.hmid = b.hmid; a.lse = b.lse; a.abar = b.abar; a.abar_layer = (size_t)c.max_batch * c.max_seq * c.max_seq;
+  a.c = b.c; a.conf = b.conf; a.pred = b.pred;
+  a.clear = b.sk_counters; a.n_clear = kCounters;
+  a.sync = reinterpret_cast<uint32_t*>(b.status) + 32; a.status = b.status;
+  return a;
+}
+// Clusters of the kernel that does a whole step, 0 where the model is not one for it.
+static int small_clusters(const d2c_ctx* ctx) {
+  const d2c_config& c = ctx->cfg;
+  const int hq_dh = c.n_q_heads * c.head_dim, qkv_out = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
+  if ((c.flags & ~D2C_FLAG_SERIAL) || c.head_dim != 64 || c.n_layers > kSmallMaxLayers || c.max_batch > kSmallMaxBatch) return 0;
+  if (c.d_model < 256 || c.d_model > 512 || hq_dh > 512 || c.d_ffn > 1024 || c.max_seq > 8192) return 0;
+  // (every CTA has columns of the products of the layers; the LM head may leave some without)
+  if (c.d_ffn < 8 * kSmallCluster || qkv_out < 16 * kSmallCluster || (long long)c.vocab * c.d_model > (1 << 20)) return 0;
+  uintptr_t low = reinterpret_cast<uintptr_t>(ctx->g_final) | reinterpret_cast<uintptr_t>(ctx->w_lm);      // (the layers' are checked; a bias may lie anywhere)
+  for (const bf16* p : ctx->bqkv) low |= reinterpret_cast<uintptr_t>(p);
+  if (low % 16) return 0;
+  const SmallArgs a = small_args(ctx, c.max_batch, c.max_seq);
+  const int most = small_step_clusters(), tiles = c.max_batch * ceil_div(c.max_seq, 16), n = most < tiles ? most : tiles;
+  if (n == 0 || n > kSmallMaxClusters || ceil_div(tiles, n) > kSmallMaxTiles || n * kSmallCluster < c.max_batch) return 0;
+  return small_step_scratch(a, n, nullptr, nullptr) <= (size_t)ctx->sk_tiles * 128 * 256 ? n : 0;
+}
+
 extern "C" {
 
 size_t d2c_workspace_bytes(const d2c_config* cfg) {
@@ -341,13 +379,14 @@ int d2c_create(const d2c_config* cfg, const d2c_weights* w, void* workspace, siz
   ctx->g_final = (const bf16*)w->g_final; ctx->w_lm = (const bf16*)w->w_lm;
   carve(*cfg, workspace, &ctx->buf);
   ctx->q_bufs = q_buffers(*cfg); ctx->sk_tiles = sk_tiles(*cfg);
+  ctx->small_clusters = small_clusters(ctx);
   {
-    bool ok = cudaHostAlloc(reinterpret_cast<void**>(&ctx->hint_host[0]), 2 * sizeof(int32_t), cudaHostAllocMapped) == cudaSuccess;
+    bool ok = cudaHostAlloc(reinterpret_cast<void**>(&ctx->hint_host[0]), 4 * sizeof(int32_t), cudaHostAllocMapped) == cudaSuccess;
     if (ok) {
-      ctx->hint_host[1] = ctx->hint_host[0] + 1;
-      ctx->hint_host[0][0] = ctx->hint_host[0][1] = 1 << 30;
+      ctx->hint_host[1] = ctx->hint_host[0] + 2;
+      ctx->hint_host[0][0] = ctx->hint_host[1][0] = 1 << 30; ctx->hint_host[0][1] = ctx->hint_host[1][1] = -1;
       ok = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->hint_dev[0]), ctx->hint_host[0], 0) == cudaSuccess;
-      ctx->hint_dev[1] = ctx->hint_dev[0] + 1;
+      ctx->hint_dev[1] = ctx->hint_dev[0] + 2;
       for (int i = 0; i < 2 && ok; ++i) ok = cudaEventCreateWithFlags(&ctx->ev_hint[i], cudaEventDisableTiming) == cudaSuccess;
     }
     if (!ok) {                                               // the step then always takes the many-row kernels
@@ -447,15 +486,97 @@ static bool stream_captures(const d2c_ctx* ctx) {
 static int previous_rows(d2c_ctx* ctx, bool capturing, int* rows) {
   const int prev = (int)(ctx->step_no & 1) ^ 1;
   if (!ctx->hint_host[0] || capturing || ctx->hint_step[prev] != ctx->step_no - 1) return D2C_OK;
+  if (ctx->hint_tagged[prev]) {
+    // (an event behind a step in one launch would come with its end, and cost the GPU 8 of 50 us between two of them)
+    const volatile uint64_t* word = reinterpret_cast<const volatile uint64_t*>(ctx->hint_host[prev]);
+    for (bool ended = false;;) {
+      for (int i = 0; i < 20000; ++i) {
+        const uint64_t v = *word;
+        if ((uint32_t)(v >> 32) == (uint32_t)ctx->hint_step[prev]) { *rows = (int)(uint32_t)v; return D2C_OK; }
+        if (ended) return D2C_OK;                              // it said nothing: like a step that was not watched
+      }
+      const cudaError_t e = cudaStreamQuery(ctx->stream);
+      if (e == cudaErrorNotReady) (void)cudaGetLastError();
+      else if (e != cudaSuccess) return cu(e);
+      else ended = true;
+    }
+  }
   const int rc = cu(cudaEventSynchronize(ctx->ev_hint[prev]));
   if (rc == D2C_OK) *rows = *reinterpret_cast<volatile int32_t*>(ctx->hint_host[prev]);
   return rc;
+}
+
+static SelectArgs select_args(const d2c_ctx* ctx, const d2c_step_args* a, bool track) {
+  const Buffers& b = ctx->buf;
+  const int L = a->seq_len;
+  SelectArgs s{};
+  s.mask = a->mask; s.conf = b.conf; s.c = a->override_c ? a->override_c : b.c; s.override_key = a->override_key;
+  s.forced = a->forced; s.forced_off = a->forced_off; s.batch = a->batch; s.seq_len = L; s.k = a->k; s.p = a->p;
+  s.stage2_candidates = ctx->cfg.stage2_candidates; s.block_lo = a->block_lo; s.block_hi = a->block_hi; s.phi_q30 = b.phi; s.phi_len = ctx->phi_len < L ? ctx->phi_len : L;
+  s.key = b.key; s.sel_idx = b.sel_idx; s.row_seq = b.row_seq; s.row_off = b.row_off; s.lm_rows = b.lm_rows;
+  s.lm_off = b.lm_off; s.slot_of_pos = b.slot_of_pos; s.rank_s = b.rank_s; s.rank_lm = b.rank_lm; s.n_b = b.n_b; s.nm_b = b.nm_b;
+  s.n_host = track ? ctx->hint_dev[ctx->step_no & 1] : nullptr;
+  return s;
+}
+// The index outputs of a step, copied by one of its kernels.
+static CopyOut index_outputs(const d2c_ctx* ctx, const d2c_step_out* out, int rows, int batch) {
+  CopyOut copies{};
+  if (out && out->sel_idx) { copies.src[0] = ctx->buf.sel_idx; copies.dst[0] = out->sel_idx; copies.n[0] = rows; }
+  if (out && out->row_off) { copies.src[1] = ctx->buf.row_off; copies.dst[1] = out->row_off; copies.n[1] = batch + 1; }
+  return copies;
+}
+// Whether a small model's step goes in one launch: while each cluster has one tile of 16 rows, and of a narrow model two, or three where
+// the rows are a part of the room only and so mostly known ones, without work for the LM head.  (us, one launch / separate kernels, one layer
+// of d 256: 61 rows of 256 positions 40 / 60, 216 of 600 56 / 71, 224 of 16 x 300 60 / 75, all of 112 rows 41 / 86, all of 224 in four
+// sequences, three tiles, 56 / 55, with 4096 columns of the LM head 71 / 58; two of d 384: 109 of 256 73 / 90, all of 112 70 / 181, 125 rows, two
+// tiles, 93 / 88; three of d 512: 106 of 600 128 / 151, 125 rows 135 / 124.)
+static bool few_for_one_launch(const d2c_ctx* ctx, int batch, int room, int rows) {
+  const d2c_config& c = ctx->cfg;
+  const int most = c.d_model > 256 || (long long)c.vocab * c.d_model > 1 << 18 ? 1 : 2 * rows <= room ? 3 : 2;
+  return batch * ceil_div(rows, 16 * batch) <= ctx->small_clusters * most;
+}
+// It is on the caller's stream.
+static int step_in_one_launch(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out, bool track) {
+  const d2c_config& c = ctx->cfg;
+  const Buffers& b = ctx->buf;
+  const int B = a->batch, L = a->seq_len, R = B * L, slot = (int)(ctx->step_no & 1);
+  SmallArgs s = small_args(ctx, B, L);
+  s.sel = select_args(ctx, a, false);
+  s.h0 = static_cast<const bf16*>(a->h0); s.h0_far = ctx->h0_far;
+  s.x = (out && out->hidden_out) ? static_cast<bf16*>(out->hidden_out) : b.x;
+  s.layer_in = out ? static_cast<bf16*>(out->layer_in) : nullptr; s.rows_cap = R;
+  s.logits = out ? out->logits : nullptr;
+  s.copies = index_outputs(ctx, out, R, B);
+  if (track) { s.n_word = reinterpret_cast<int2*>(ctx->hint_dev[slot]); s.n_tag = (int)ctx->step_no; }
+  small_step_scratch(s, ctx->small_clusters, b.sk_partials, &s);
+  D2C_TRY(ctx, launch_small_step(s, ctx->small_clusters, ctx->stream));
+  if (track) { ctx->hint_step[slot] = ctx->step_no; ctx->hint_tagged[slot] = true; }
+  ctx->step_no++;
+  if (ctx->early_hidden_host && ctx->copy_stream) {           // d2c_step_host's rows
+    if (ctx->early_hidden_dev) { D2C_TRY(ctx, launch_rows_to_host(s.x, b.row_off + B, c.d_model, ctx->early_hidden_dev, ctx->stream)); }
+    else D2C_TRY(ctx, cu(cudaMemcpyAsync(ctx->early_hidden_host, s.x, (size_t)R * c.d_model * sizeof(bf16), cudaMemcpyDeviceToHost, ctx->stream)));
+  }
+  return D2C_OK;
 }
 
 int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   D2C_TRY(ctx, check_step_args(ctx, a));
   const d2c_config& c = ctx->cfg;
   const Buffers& b = ctx->buf;
+  {
+    const void* x = (out && out->hidden_out) ? out->hidden_out : b.x;
+    if (reinterpret_cast<uintptr_t>(x) % 16 || reinterpret_cast<uintptr_t>(a->h0) % 16)
+      return fail(ctx, D2C_EINVAL, "d2c_step: h0 and hidden_out must be 16-byte aligned");
+  }
+  if (ctx->small_clusters > 0 && !ctx->prof && !(out && reinterpret_cast<uintptr_t>(out->layer_in) % 16)) {
+    // One launch where few rows are expected, going by the step before like everything here, or where there is room for no more.
+    const int rows = a->batch * a->seq_len;
+    const bool capturing = stream_captures(ctx), any = few_for_one_launch(ctx, a->batch, rows, rows);
+    const bool track = ctx->hint_host[0] != nullptr && !capturing && (!any || ctx->host_call);
+    int expect = rows;
+    if (!any) D2C_TRY(ctx, previous_rows(ctx, capturing, &expect));
+    if (few_for_one_launch(ctx, a->batch, rows, expect)) return step_in_one_launch(ctx, a, out, track);
+  }
   // critical path on `st`, probabilities + rollout on `side` (the same stream while profiling or when serial)
   const int B = a->batch, L = a->seq_len, R = B * L, d = c.d_model;
   // Whether a product's weights alone give all SMs work, with one tile of tokens and whichever kernel takes it.  (By the tiles of all
@@ -532,21 +653,12 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   const int qkv_out = (hq + 2 * hkv) * dh;
   const size_t cache_layer = (size_t)c.max_batch * c.max_seq * hkv * dh;
   bf16* x = (out && out->hidden_out) ? static_cast<bf16*>(out->hidden_out) : b.x;
-  if (reinterpret_cast<uintptr_t>(x) % 16 || reinterpret_cast<uintptr_t>(a->h0) % 16)
-    return fail(ctx, D2C_EINVAL, "d2c_step: h0 and hidden_out must be 16-byte aligned");
 
-  SelectArgs s{};
-  s.mask = a->mask; s.conf = b.conf; s.c = a->override_c ? a->override_c : b.c; s.override_key = a->override_key;
-  s.forced = a->forced; s.forced_off = a->forced_off; s.batch = B; s.seq_len = L; s.k = a->k; s.p = a->p;
-  s.stage2_candidates = c.stage2_candidates; s.block_lo = a->block_lo; s.block_hi = a->block_hi; s.phi_q30 = b.phi; s.phi_len = ctx->phi_len < L ? ctx->phi_len : L;
-  s.key = b.key; s.sel_idx = b.sel_idx; s.row_seq = b.row_seq; s.row_off = b.row_off; s.lm_rows = b.lm_rows;
-  s.lm_off = b.lm_off; s.slot_of_pos = b.slot_of_pos; s.rank_s = b.rank_s; s.rank_lm = b.rank_lm; s.n_b = b.n_b; s.nm_b = b.nm_b;
-  s.n_host = track ? ctx->hint_dev[slot] : nullptr;
   D2C_TRY(ctx, mark(ctx, PH_SELECT));
-  D2C_TRY(ctx, launch_select(s, st));
+  D2C_TRY(ctx, launch_select(select_args(ctx, a, track), st));
   if (track) {
     D2C_TRY(ctx, cu(cudaEventRecord(ctx->ev_hint[slot], st)));
-    ctx->hint_step[slot] = ctx->step_no;
+    ctx->hint_step[slot] = ctx->step_no; ctx->hint_tagged[slot] = false;
   }
   ctx->step_no++;
   const int32_t* n_rows = b.row_off + B;
@@ -799,9 +911,7 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   gl.st_max = b.st_max; gl.st_sum = b.st_sum; gl.st_arg = b.st_arg; gl.n_tiles = lm_tiles(c.vocab);
   gl.logits = out ? out->logits : nullptr;
   D2C_TRY(ctx, gemm(ctx, gl, EPI_LMSTATS));
-  CopyOut copies{};                                    // the index outputs leave with the last kernel of the chain
-  if (out && out->sel_idx) { copies.src[0] = b.sel_idx; copies.dst[0] = out->sel_idx; copies.n[0] = R; }
-  if (out && out->row_off) { copies.src[1] = b.row_off; copies.dst[1] = out->row_off; copies.n[1] = B + 1; }
+  const CopyOut copies = index_outputs(ctx, out, R, B);      // they leave with the last kernel of the chain
   D2C_TRY(ctx, launch_lm_reduce(b.st_max, b.st_sum, b.st_arg, gl.n_tiles, n_lm, R, b.lm_rows, b.sel_idx, b.row_seq, L, b.conf, b.pred, copies, b.sk_counters + 2 * kSkMaxTiles, 2 * kPairCounters, st));
   if (pass_left) {
     D2C_TRY(ctx, cu(cudaStreamWaitEvent(side, ctx->ev_fwd, 0)));
@@ -894,8 +1004,9 @@ static int enqueue_step_host(d2c_ctx* ctx, const d2c_step_args* h, const d2c_hos
   ctx->early_hidden_host = early ? out->hidden_out_host : nullptr;
   ctx->early_hidden_dev = early && few_expected ? mapped(out->hidden_out_host, R * c.d_model * sizeof(bf16)) : nullptr;
   if (reinterpret_cast<uintptr_t>(ctx->early_hidden_dev) % 16) ctx->early_hidden_dev = nullptr;
+  ctx->host_call = true; ctx->h0_far = a.h0 != b.h0_stage;
   const int step_rc = d2c_step(ctx, &a, &dev_out);
-  ctx->early_hidden_host = ctx->early_hidden_dev = nullptr;
+  ctx->early_hidden_host = ctx->early_hidden_dev = nullptr; ctx->host_call = ctx->h0_far = false;
   if (step_rc != D2C_OK) return step_rc;
   // every other result is copied without knowing the row count (worst-case sizes), then one synchronisation
   if (out) {
