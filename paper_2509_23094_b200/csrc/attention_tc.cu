@@ -60,7 +60,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, rows, split_last; };      // group: query heads of a K/V head; rows: selected rows of a query tile
+struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, rows, split_last, places; };      // group: query heads of a K/V head; rows: selected rows of a query tile; places: tiles of a sequence's head that the grid has places for (0: numbered in turn)
 
 // ------------------------------------------------------------------------------------------------
 // Forward kernel.  One CTA owns up to 256 selected rows of one (sequence, head): two query tiles of
@@ -131,7 +131,7 @@ __device__ __forceinline__ int lane_of_item(int mine, int& i) {
 // 49.0, 300 of five x 3071 x 32 144.4 -> 133.0, 2880 of two x 4096 348.5 -> 345.5, 976 of four x 1536 and 797 x 797 no difference.  (Items
 // of two tiles first, those of one behind them: 142 where it is 134, as a head's keys then come out of the L2 no longer.)
 template <bool kGroup, bool kSplitLast>
-__device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int heads, int rows_, int sm_count) {
+__device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int heads, int rows_, int sm_count, int places) {
   const int rows = kGroup ? rows_ : AQ;
   const int lane = threadIdx.x & 31;
   int i = blockIdx.x, all = 0, pairs = 0, half = -1;                // tiles, and pairs of them
@@ -143,6 +143,12 @@ __device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int
     const int whole = div24(pairs, sm_count) * sm_count;
     if (all > sm_count && 2 * (pairs - whole) <= sm_count && i >= whole) { half = (i - whole) & 1; i = whole + ((i - whole) >> 1); }
   };
+  // (where there is room for one tile each of `places` tiles a head, all of them run at once, wherever they stand: without the numbering
+  // 0.5 us of a launch)
+  if (!kSplitLast && places > 0) {
+    const int bg = div24(i, places), b = div24(bg, heads), first = row_off[b], r = (i - bg * places) * rows;
+    return make_int4(b, bg - b * heads, first + r, min(rows, row_off[b + 1] - first - r));
+  }
   const auto item_of = [&](int b, int g, int first, int n, int r, int width) {
     if (kSplitLast && half >= 0) { r += half * rows; width = 1; }
     return make_int4(b, g, first + r, min(width * rows, n - r));
@@ -194,15 +200,15 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   __shared__ int s_item[4];
   volatile int* item = s_item;
   if constexpr (kSplit) {
-    // The row tile is the slowest index, so that the live ones start first.  The grid has room for half of the tiles that there can be:
-    // with more rows than that every CTA takes two.  (Its other CTAs find nothing to do.)
+    // The row tile is the slowest index, so that the live ones start first.  The grid may have room for half of the tiles only that there can
+    // be: with more rows than that every CTA takes two.  (Its other CTAs find nothing to do.)
     const int b = (int)blockIdx.z % a.batch, r0 = a.row_off[b], nb = a.row_off[b + 1] - r0;
-    const int width = nb > (int)gridDim.z / a.batch * tile_rows ? 2 * tile_rows : tile_rows, at = (int)blockIdx.z / a.batch * width;
+    const int width = nb > p.places * tile_rows ? 2 * tile_rows : tile_rows, at = (int)blockIdx.z / a.batch * width;
     if (at >= nb) return;                                           // uniform in the cluster: nothing allocated yet
     if (threadIdx.x == 0) { item[0] = b; item[1] = blockIdx.y; item[2] = r0 + at; item[3] = min(width, nb - at); }
   } else if (warp == 0) {
-    const int4 it = p.split_last ? forward_item<kGroup, true>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count)
-                                 : forward_item<kGroup, false>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count);
+    const int4 it = p.split_last ? forward_item<kGroup, true>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count, 0)
+                                 : forward_item<kGroup, false>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count, p.places);
     if (lane == 0) { item[0] = it.x; item[1] = it.y; item[2] = it.z; item[3] = it.w; }
   }
   const int L = a.seq_len, tiles = (L + AKEYS - 1) / AKEYS;
@@ -995,7 +1001,7 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   // rows of seven heads, where a head's own rows filled their last tile only in part.  Forward alone, a head's rows / a group's, us, 28 heads
   // over 4: 260 rows of eight sequences x 700 keys 48.6 / 33.6, 147 of four x 1187 24.5 / 21.2, 976 of four x 1536 100.4 / 93.6.
   const int group = a.hq / a.hkv, tile_rows = AQ / group;
-  AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, tile_rows, 0};
+  AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, tile_rows, 0, 0};
   const int rows_seq = expected_rows_per_seq(a);
   if (a.which != 2) {
     static PerDevice attr_set;
@@ -1023,12 +1029,15 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
       if (s * units <= sms - 16 && key_tiles >= (s == 4 ? 16 : s + 1)) p.splits = s;
     cudaLaunchConfig_t cfg = {};
     const int xtiles = ceil_div(a.max_rows_per_seq, tile_rows);
-    // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond; with shared keys clusters for half of the
-    // tiles, which take two each where that is not enough: 32 layers at 80 rows of 768 positions 3810 -> 3775 us against one for each)
+    // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond; with shared keys, where no more than half of
+    // the tiles are expected, clusters for half of them, which take two each where that is not enough: 32 layers at 80 rows of 768 positions
+    // 3810 -> 3775 us against one for each, but two of d 512, all of 521 rows, 128 -> 134)
     const int most = a.hkv * a.batch * ((xtiles + 1) / 2), single = a.hkv * a.batch * xtiles < sms ? a.hkv * a.batch * xtiles : sms;
+    const int clusters = 2 * ceil_div(rows_seq, tile_rows) > xtiles ? xtiles : (xtiles + 1) / 2;
+    p.places = p.splits > 1 ? clusters : a.hkv * a.batch * xtiles <= sms ? xtiles : 0;
     const int pairs = ceil_div(ceil_div(rows_seq, tile_rows), 2) * a.hkv * a.batch;      // (expected; where none are to be split, looking for them costs 0.4 us)
     p.split_last = units > sms && pairs > sms && pairs % sms > 0 && 2 * (pairs % sms) <= sms;
-    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hkv, (xtiles + 1) / 2 * a.batch) : dim3((most > single ? most : single) + (p.split_last ? sms / 2 : 0));
+    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hkv, clusters * a.batch) : dim3((most > single ? most : single) + (p.split_last ? sms / 2 : 0));
     cfg.blockDim = dim3(FWD_THREADS); cfg.dynamicSmemBytes = smem_fwd; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
