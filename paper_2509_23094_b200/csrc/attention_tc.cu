@@ -60,7 +60,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, rows, split_last, places; };      // group: query heads of a K/V head; rows: selected rows of a query tile; places: tiles of a sequence's head that the grid has places for (0: numbered in turn)
+struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, heads, kv_share, rows, split_last, places; };      // group: query heads of a tile, of the same K/V head; heads: such groups; kv_share: those of a K/V head; rows: selected rows of a query tile; places: tiles of a sequence's head that the grid has places for (0: numbered in turn)
 
 // ------------------------------------------------------------------------------------------------
 // Forward kernel.  One CTA owns up to 256 selected rows of one (sequence, head): two query tiles of
@@ -131,7 +131,7 @@ __device__ __forceinline__ int lane_of_item(int mine, int& i) {
 // 49.0, 300 of five x 3071 x 32 144.4 -> 133.0, 2880 of two x 4096 348.5 -> 345.5, 976 of four x 1536 and 797 x 797 no difference.  (Items
 // of two tiles first, those of one behind them: 142 where it is 134, as a head's keys then come out of the L2 no longer.)
 template <bool kGroup, bool kSplitLast>
-__device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int heads, int rows_, int sm_count, int places) {
+__device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int heads, int rows_, int sm_count) {
   const int rows = kGroup ? rows_ : AQ;
   const int lane = threadIdx.x & 31;
   int i = blockIdx.x, all = 0, pairs = 0, half = -1;                // tiles, and pairs of them
@@ -143,12 +143,6 @@ __device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int
     const int whole = div24(pairs, sm_count) * sm_count;
     if (all > sm_count && 2 * (pairs - whole) <= sm_count && i >= whole) { half = (i - whole) & 1; i = whole + ((i - whole) >> 1); }
   };
-  // (where there is room for one tile each of `places` tiles a head, all of them run at once, wherever they stand: without the numbering
-  // 0.5 us of a launch)
-  if (!kSplitLast && places > 0) {
-    const int bg = div24(i, places), b = div24(bg, heads), first = row_off[b], r = (i - bg * places) * rows;
-    return make_int4(b, bg - b * heads, first + r, min(rows, row_off[b + 1] - first - r));
-  }
   const auto item_of = [&](int b, int g, int first, int n, int r, int width) {
     if (kSplitLast && half >= 0) { r += half * rows; width = 1; }
     return make_int4(b, g, first + r, min(width * rows, n - r));
@@ -182,7 +176,7 @@ __device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int
   return make_int4(0, 0, 0, 0);
 }
 
-// kGroup: a K/V head has several query heads (one: the tile's divisions by their number fold away, 0.3 us of a CTA).
+// kGroup: a tile has several query heads (one: the tile's divisions by their number fold away, 0.3 us of a CTA).
 template <bool kSplit, bool kGroup>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -206,9 +200,15 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     const int width = nb > p.places * tile_rows ? 2 * tile_rows : tile_rows, at = (int)blockIdx.z / a.batch * width;
     if (at >= nb) return;                                           // uniform in the cluster: nothing allocated yet
     if (threadIdx.x == 0) { item[0] = b; item[1] = blockIdx.y; item[2] = r0 + at; item[3] = min(width, nb - at); }
+  } else if (p.places > 0) {
+    // (by its place among `places` of each head where all places run at once: the numbering takes a CTA of several sequences 0.5 us)
+    const int bg = div24(blockIdx.x, p.places), b = div24(bg, p.heads), r0 = a.row_off[b], at = ((int)blockIdx.x - bg * p.places) * tile_rows;
+    const int nrows = min(tile_rows, a.row_off[b + 1] - r0 - at);
+    if (nrows <= 0) return;
+    if (threadIdx.x == 0) { item[0] = b; item[1] = bg - b * p.heads; item[2] = r0 + at; item[3] = nrows; }
   } else if (warp == 0) {
-    const int4 it = p.split_last ? forward_item<kGroup, true>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count, 0)
-                                 : forward_item<kGroup, false>(a.row_off, a.batch, a.hkv, tile_rows, p.sm_count, p.places);
+    const int4 it = p.split_last ? forward_item<kGroup, true>(a.row_off, a.batch, p.heads, tile_rows, p.sm_count)
+                                 : forward_item<kGroup, false>(a.row_off, a.batch, p.heads, tile_rows, p.sm_count);
     if (lane == 0) { item[0] = it.x; item[1] = it.y; item[2] = it.z; item[3] = it.w; }
   }
   const int L = a.seq_len, tiles = (L + AKEYS - 1) / AKEYS;
@@ -251,11 +251,16 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (warp < 4) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
   if (warp == 0) {
     if (lane == 0) {
-      const int g = item[1], r0 = item[2], kv_row0 = item[0] * a.cache_seq + first * AKEYS;
+      const int h = item[1], g = kGroup || p.kv_share == 1 ? h : h / p.kv_share, r0 = item[2], kv_row0 = item[0] * a.cache_seq + first * AKEYS;
       mbar_expect_tx(B(0), nq * tile_rows * group * ADH * 2);
       for (int q = 0; q < nq; ++q) {
-        tma_load_3d(sQ(q), &tmQ, 0, g * group, r0 + q * tile_rows, B(0));
-        tma_load_3d(sQ(q) + HALF_BYTES, &tmQ, 64, g * group, r0 + q * tile_rows, B(0));
+        if constexpr (kGroup) {
+          tma_load_3d(sQ(q), &tmQ, 0, h * group, r0 + q * tile_rows, B(0));
+          tma_load_3d(sQ(q) + HALF_BYTES, &tmQ, 64, h * group, r0 + q * tile_rows, B(0));
+        } else {
+          tma_load_2d(sQ(q), &tmQ, h * ADH, r0 + q * AQ, B(0));
+          tma_load_2d(sQ(q) + HALF_BYTES, &tmQ, h * ADH + 64, r0 + q * AQ, B(0));
+        }
       }
       int issued = 0;
       for (int j = 0; j < T; ++j) {
@@ -1000,9 +1005,22 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   // A query tile holds the rows of all query heads of a K/V head, (row, head) by (row, head), as many whole rows as there is room for: 18
   // rows of seven heads, where a head's own rows filled their last tile only in part.  Forward alone, a head's rows / a group's, us, 28 heads
   // over 4: 260 rows of eight sequences x 700 keys 48.6 / 33.6, 147 of four x 1187 24.5 / 21.2, 976 of four x 1536 100.4 / 93.6.
-  const int group = a.hq / a.hkv, tile_rows = AQ / group;
-  AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, tile_rows, 0, 0};
-  const int rows_seq = expected_rows_per_seq(a);
+  // Not where a head's tiles by themselves are few enough for as many CTAs to share their keys: the tiles then have fewer rows to finish with
+  // (four layers, 18 rows x 600, 28 heads over 4, 644 / 630 us; 28 rows x 1390 671 / 659).
+  const int rows_seq = expected_rows_per_seq(a), key_tiles = ceil_div(a.seq_len, AKEYS);
+  // Few tiles (expected): 2 to 4 CTAs share a tile's keys while all of them still run at once.  Four only
+  // for many key tiles: measured alone at 32 heads (us, 1 / 2 / 3 / 4 CTAs) 768 keys 20.4 / 18.4 / 16.4 / 17.3,
+  // 2048 keys 36.8 / 27.6 / 24.6 / 22.5, 4096 keys 64.4 / 43.0 / 36.8 / 31.7.
+  auto splits_of = [&](int units) {
+    int splits = 1;
+    for (int s = 2; s <= kMaxSplits; ++s)
+      if (s * units <= sms - 16 && key_tiles >= (s == 4 ? 16 : s + 1)) splits = s;
+    return splits;
+  };
+  const int solo = splits_of(ceil_div(rows_seq, AQ) * a.hq * a.batch), packed = AQ / (a.hq / a.hkv);
+  const bool pack = solo == 1 || solo < splits_of(ceil_div(rows_seq, packed) * a.hkv * a.batch);
+  const int group = pack ? a.hq / a.hkv : 1, heads = a.hq / group, tile_rows = AQ / group;
+  AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, heads, a.hq / a.hkv / group, tile_rows, 0, 0};
   if (a.which != 2) {
     static PerDevice attr_set;
     if (attr_set.first()) {
@@ -1013,31 +1031,31 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     bool made = false;
     if (a.cache[0]) {
       m = reinterpret_cast<Maps*>(a.cache[0]->maps);
-      made = a.cache[0]->same(a.q, a.kc, a.vc, a.q_rows, a.hq, a.ldq, (long long)kv_rows, (long long)kv_cols, 3);
+      made = a.cache[0]->same(a.q, a.kc, a.vc, a.q_rows, a.hq, a.ldq, (long long)kv_rows, (long long)kv_cols, 3 + 8 * group);
     }
     if (!made) {
-      int rc = make_bf16_head_map(&m->q, a.q, (uint64_t)a.q_rows, (uint64_t)a.hq, (uint64_t)a.ldq, (uint32_t)tile_rows, (uint32_t)group);
+      // (one head a tile: rows by columns; as boxes of (row, head) they come in 0.25 us later)
+      int rc = group == 1 ? make_bf16_map(&m->q, a.q, (uint64_t)a.q_rows, (uint64_t)a.hq * a.dh, (uint64_t)a.ldq, AQ)
+                          : make_bf16_head_map(&m->q, a.q, (uint64_t)a.q_rows, (uint64_t)a.hq, (uint64_t)a.ldq, (uint32_t)tile_rows, (uint32_t)group);
       if (rc == D2C_OK) rc = make_bf16_map(&m->k, a.kc, kv_rows, kv_cols, kv_cols, 128);
       if (rc == D2C_OK) rc = make_bf16_map(&m->v, a.vc, kv_rows, kv_cols, kv_cols, 128);
       if (rc != D2C_OK) { if (a.cache[0]) a.cache[0]->forget(); return rc; }
     }
-    // Few tiles of 128 rows (expected): 2 to 4 CTAs share a tile's keys while all of them still run at once.  Four only
-    // for many key tiles: measured alone at 32 heads (us, 1 / 2 / 3 / 4 CTAs) 768 keys 20.4 / 18.4 / 16.4 / 17.3,
-    // 2048 keys 36.8 / 27.6 / 24.6 / 22.5, 4096 keys 64.4 / 43.0 / 36.8 / 31.7.
-    const int units = ceil_div(rows_seq, tile_rows) * a.hkv * a.batch, key_tiles = ceil_div(a.seq_len, AKEYS);
-    for (int s = 2; s <= kMaxSplits; ++s)
-      if (s * units <= sms - 16 && key_tiles >= (s == 4 ? 16 : s + 1)) p.splits = s;
+    const int units = ceil_div(rows_seq, tile_rows) * heads * a.batch;
+    p.splits = splits_of(units);
     cudaLaunchConfig_t cfg = {};
     const int xtiles = ceil_div(a.max_rows_per_seq, tile_rows);
     // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond; with shared keys, where no more than half of
     // the tiles are expected, clusters for half of them, which take two each where that is not enough: 32 layers at 80 rows of 768 positions
     // 3810 -> 3775 us against one for each, but two of d 512, all of 521 rows, 128 -> 134)
-    const int most = a.hkv * a.batch * ((xtiles + 1) / 2), single = a.hkv * a.batch * xtiles < sms ? a.hkv * a.batch * xtiles : sms;
+    const int most = heads * a.batch * ((xtiles + 1) / 2), single = heads * a.batch * xtiles < sms ? heads * a.batch * xtiles : sms;
     const int clusters = 2 * ceil_div(rows_seq, tile_rows) > xtiles ? xtiles : (xtiles + 1) / 2;
-    p.places = p.splits > 1 ? clusters : a.hkv * a.batch * xtiles <= sms ? xtiles : 0;
-    const int pairs = ceil_div(ceil_div(rows_seq, tile_rows), 2) * a.hkv * a.batch;      // (expected; where none are to be split, looking for them costs 0.4 us)
+    const int pairs = ceil_div(ceil_div(rows_seq, tile_rows), 2) * heads * a.batch;      // (expected; where none are to be split, looking for them costs 0.4 us)
     p.split_last = units > sms && pairs > sms && pairs % sms > 0 && 2 * (pairs % sms) <= sms;
-    cfg.gridDim = p.splits > 1 ? dim3(p.splits, a.hkv, clusters * a.batch) : dim3((most > single ? most : single) + (p.split_last ? sms / 2 : 0));
+    // By place where all places run at once: two layers of d 512, all rows of eight sequences of 300, 179.7 -> 177.8 us a step.
+    const bool by_place = p.splits == 1 && single < sms;
+    p.places = p.splits > 1 ? clusters : by_place ? xtiles : 0;
+    cfg.gridDim = p.splits > 1 ? dim3(p.splits, heads, clusters * a.batch) : by_place ? dim3(single) : dim3((most > single ? most : single) + (p.split_last ? sms / 2 : 0));
     cfg.blockDim = dim3(FWD_THREADS); cfg.dynamicSmemBytes = smem_fwd; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1075,7 +1093,8 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   // 300 rows of five sequences x 3071 keys 100.5 -> 95.8 us, 147 of four x 1187 32.4 -> 31.1, 420 of three x 1100 38.3 -> 37.8.  Finding its
   // number takes a cluster up to 0.9 us, which it is not worth with fewer (260 of eight x 700 41.8 / 42.7) or one sequence.
   const int xs = 2 * p.head_groups * ceil_div(a.seq_len, 2 * AKEYS), worst_tiles = ceil_div(a.max_rows_per_seq, p.row_tile);
-  const bool in_turn = a.batch > 1 && worst_tiles >= 2 * ceil_div(rows_seq, p.row_tile);
+  const int empty = xs * a.batch * (worst_tiles - ceil_div(rows_seq, p.row_tile));
+  const bool in_turn = a.batch > 1 && worst_tiles >= 2 * ceil_div(rows_seq, p.row_tile) && empty > 2 * sms;
   cfg.gridDim = p.pairs > 0 ? dim3(2 * p.pairs) : (in_turn ? dim3(xs * worst_tiles * a.batch) : dim3(xs, worst_tiles, a.batch));
   cfg.blockDim = dim3(ABAR_THREADS); cfg.dynamicSmemBytes = kAbarSmem; cfg.stream = st;
   cudaLaunchAttribute attr[2];
