@@ -15,7 +15,7 @@
 // the L2 into fragments.  Both are read 16 bytes a lane: the order of K inside a product is free, so lane q of a group of four takes
 // eight neighbouring elements of a row, and two MMAs' fragments are the two halves of what it has.
 //
-// Measured (us a step, this launch / the separate kernels; one layer of d 256, 94 rows of 128 positions: 41 / 58): 256 threads a CTA
+// Measured (us a step, this launch / the separate kernels; one layer of d 256, 94 rows of 128 positions: 41 / 52): 256 threads a CTA
 // 41, 512 52 (barriers; half of the instructions are per warp); rows by bulk copies 2 a product more than by cp.async; a normed row
 // pushed into the other CTAs' shared memory 44; keys of a unit shared by several CTAs and merged: 0 to 9 more up to 2100 positions, 2 to 8 %
 // less at 4096; heads of 128, which need twice the registers for V and Q: 5 to 15 % ahead of the separate kernels up to 130 rows only, so left to them.
