@@ -201,7 +201,8 @@ typedef struct {
 int d2c_state_ptrs(d2c_ctx* ctx, d2c_state* out);
 
 /* Synchronises the stream and returns the device status word's error code (D2C_OK, or what a kernel's
- * bounded wait recorded: D2C_ETIMEOUT with the wait's site number in the error text).  The word is sticky:
+ * bounded wait recorded: D2C_ETIMEOUT with the wait's site number in the error text; D2C_ECUDA at site 63 if a
+ * kernel found itself launched in other clusters than its own, and did nothing).  The word is sticky:
  * it keeps the first error until the caller writes zeros to status[0..3]. */
 int d2c_sync_status(d2c_ctx* ctx);
 

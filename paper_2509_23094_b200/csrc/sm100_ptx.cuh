@@ -168,6 +168,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 }
 // ------------------------------------------------------------------------------------------- pairs of CTAs (cta_group::2)
 constexpr uint32_t kPeerMask = 0xFEFFFFFFu;                   // clears the CTA-rank bit of a shared::cluster address: the even CTA
+__device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ uint32_t cluster_ctarank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ void cluster_arrive_all() { asm volatile("barrier.cluster.arrive.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }   // orders no memory

@@ -108,7 +108,9 @@ __device__ __forceinline__ int quot(int a, int b) {
 // The products of a step: four of each layer, and the LM head.
 enum Step { S_QKV = 0, S_O = 1, S_GATEUP = 2, S_DOWN = 3, S_LM = 4 };
 
-__global__ void __launch_bounds__(NT, 1) small_step_kernel(const __grid_constant__ SmallArgs a) {
+// The cluster's size is the kernel's own, not an attribute of its launch: a tool that launches the kernel in its own way (ncu) kept the
+// cooperative attribute and left that one out, and clusters of one CTA meet every barrier and write a sixteenth of the results.
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_kernel(const __grid_constant__ SmallArgs a) {
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ int s_off[MAXB + 1], s_lmoff[MAXB + 1], s_toff[MAXB + 1], s_ct[kSmallMaxClusters + 1];
   __shared__ int4 s_tile[MAXT];                    // first row, rows, sequence, first row of the sequence's cache
@@ -122,6 +124,11 @@ __global__ void __launch_bounds__(NT, 1) small_step_kernel(const __grid_constant
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, q = lane & 3;
   const int rank = (int)cluster_ctarank(), cidx = blockIdx.x / CL, ncl = gridDim.x / CL;
   const int B = a.sel.batch, L = a.sel.seq_len, d = a.d, hq = a.hq, n_layers = a.n_layers;
+  // (in another cluster nothing is begun: all CTAs leave, and the status tells)
+  if (cluster_size() != CL) {
+    if (blockIdx.x == 0 && tid == 0 && atomicCAS(a.status, 0, D2C_ECUDA) == 0) { a.status[1] = 63; a.status[2] = (int)cluster_size(); }
+    return;
+  }
   constexpr int UH = DH / 16;                      // units of a head: eight columns of its low half, eight of its high half
   const int d_o = hq * DH, kv_ld = a.hkv * DH;
   unsigned char* s_gain = dyn;
@@ -830,10 +837,8 @@ int config(int clusters, cudaStream_t st, cudaLaunchConfig_t* cfg, cudaLaunchAtt
     D2C_CUDA_OK(cudaFuncSetAttribute(small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem));
   }
   cfg->gridDim = dim3(clusters * CL); cfg->blockDim = dim3(NT); cfg->dynamicSmemBytes = kSmallSmem; cfg->stream = st;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeCooperative; attr[1].val.cooperative = 1;
-  cfg->attrs = attr; cfg->numAttrs = 2;
+  attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
+  cfg->attrs = attr; cfg->numAttrs = 1;
   return D2C_OK;
 }
 }  // namespace
@@ -844,7 +849,7 @@ int small_step_clusters() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
   if (known[dev]) return known[dev] - 1;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   if (config(1, nullptr, &cfg, attr) != D2C_OK || cudaOccupancyMaxActiveClusters(&n, small_step_kernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
   known[dev] = n + 1;
   return n;
@@ -862,7 +867,7 @@ size_t small_step_scratch(const SmallArgs& a, int clusters, float* base, SmallAr
 
 int launch_small_step(const SmallArgs& a, int clusters, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   const int rc = config(clusters, st, &cfg, attr);
   if (rc != D2C_OK) return rc;
   D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, small_step_kernel, a));

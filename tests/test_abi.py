@@ -31,6 +31,22 @@ def test_every_declared_symbol_is_exported(lib):
     assert sorted(binding.SYMBOLS) == names
 
 
+def test_cooperative_kernels_have_clusters_of_their_own():
+    """A kernel that is launched cooperatively and goes by its rank in a cluster states the cluster's size in its declaration and looks
+    at what it got: as an attribute of the launch the size does not reach every launch (ncu leaves it out), and no barrier tells."""
+    found = 0
+    for name in os.listdir(build.CSRC):
+        text = open(os.path.join(build.CSRC, name)).read()
+        if "cudaLaunchAttributeCooperative" not in text:
+            continue
+        assert "cudaLaunchAttributeClusterDimension" not in text, name
+        for kernel in re.findall(r"__global__.*?\{", text, flags=re.S):
+            assert re.search(r"__cluster_dims__\(CL, 1, 1\)", kernel), (name, kernel)
+            found += 1
+        assert "cluster_size() != CL" in text, name
+    assert found == 1
+
+
 def test_workspace_bytes_and_config_validation(lib):
     cfg = binding.make_config(inputs.TOY, 1, 128)
     small = binding.d2c_workspace_bytes(cfg)
