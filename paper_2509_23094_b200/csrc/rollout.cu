@@ -128,6 +128,7 @@ __global__ void __cluster_dims__(kRolloutCluster, 1, 1) __launch_bounds__(32 * k
     }
   };
   request();
+  __syncwarp();
   cluster_sync_all();                                          // the others have started; this CTA's arrays are set
   for (int l = a.n_layers - 1; l >= 0; --l) {
     const float* uc = u[(a.n_layers - 1 - l) & 1];
@@ -172,6 +173,7 @@ __global__ void __cluster_dims__(kRolloutCluster, 1, 1) __launch_bounds__(32 * k
         }
       }
     }
+    __syncwarp();
     if (l > 0) cluster_sync_all();                             // u is whole everywhere; part and the old u may be written again
   }
 }

@@ -67,8 +67,9 @@ __device__ __forceinline__ void copy16(void* to, const void* from) {
 __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---- barriers ----------------------------------------------------------------------------------
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// (.aligned: all threads of a warp together.  Most of them come out of loops whose trip counts differ inside a warp.)
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // All CTAs of the grid, which a cooperative launch keeps on the GPU together.  The wait is bounded: behind one that gave up the CTA
 // goes on without waiting (every index that it takes from memory is kept inside its buffers), so all barriers are still reached,

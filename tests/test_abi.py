@@ -47,6 +47,20 @@ def test_cooperative_kernels_have_clusters_of_their_own():
     assert found == 1
 
 
+def test_aligned_cluster_barriers_stand_behind_a_meeting_of_the_warp():
+    """barrier.cluster with .aligned wants all threads of a warp at the same instruction; behind a loop whose trip count differs between
+    them nothing says that they are.  So __syncwarp() stands right before it, or before the call of the function that holds it."""
+    asked = re.compile(r"cluster_(sync_all|arrive_all|arrive_relaxed)\(\);|barrier\.cluster\.arrive\.release\.aligned")
+    found = 0
+    for name in sorted(os.listdir(build.CSRC)):
+        lines = open(os.path.join(build.CSRC, name)).read().split("\n")
+        for i, line in enumerate(lines):
+            if asked.search(line) and not line.startswith("__device__ __forceinline__ void cluster_sync_all"):
+                assert any("__sync" in before for before in lines[max(i - 2, 0):i + 1]), (name, i + 1)
+                found += 1
+    assert found >= 10
+
+
 def test_workspace_bytes_and_config_validation(lib):
     cfg = binding.make_config(inputs.TOY, 1, 128)
     small = binding.d2c_workspace_bytes(cfg)
