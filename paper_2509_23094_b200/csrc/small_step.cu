@@ -72,10 +72,10 @@ __device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("b
 __device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // All CTAs of the grid, which a cooperative launch keeps on the GPU together.  The wait is bounded: behind one that gave up the CTA
-// goes on without waiting (every index that it takes from memory is kept inside its buffers), so all barriers are still reached,
-// and the step's status tells.
+// goes on without waiting, so all barriers are still reached, and the step's status tells.  Behind the first, which all others' indices
+// come from, it has no rows and takes no index from memory; what later ones let through are values.
 struct Grid {
-  uint32_t* count; int* status; uint32_t due; bool dead;
+  uint32_t* count; int* status; uint32_t due; bool dead;             // dead: in thread 0
   __device__ __forceinline__ void arrive() {
     __syncthreads();
     if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
@@ -202,7 +202,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
   // ---- the rows of this cluster ----------------------------------------------------------------------
   if (warp == 0) {
     int n = 0, m = 0;
-    if (lane < B) { n = min(max(__ldcg(a.sel.n_b + lane), 0), L); m = min(max(__ldcg(a.sel.nm_b + lane), 0), n); }
+    const bool lost = __shfl_sync(0xffffffffu, grid.dead, 0);      // nothing is known of the selection
+    if (lane < B && !lost) { n = min(max(__ldcg(a.sel.n_b + lane), 0), L); m = min(max(__ldcg(a.sel.nm_b + lane), 0), n); }
     int t = (n + 15) >> 4, sn = n, sm = m, st = t;
 #pragma unroll 1
     for (int o = 1; o < B; o <<= 1) {

@@ -109,6 +109,44 @@ def test_counts_left_by_a_wait_that_gave_up_do_not_reach_the_next_step():
             assert all(torch.equal(a, b) for a, b in zip(other, runs[1]))
 
 
+def test_a_small_step_whose_grid_never_meets_has_no_rows_and_says_so():
+    """A counter that starts far below what the CTAs of a one-launch step add to it: their first wait runs out (2 s), none of them takes an
+    index from the memory that it waited for, so there are no rows and nothing of the state changes, the status tells, and the step behind
+    it finds the counters at zero again."""
+    wl = inputs.WORKLOADS["toy"]
+    pair = Pair(wl)
+    shape, seq, d = wl.shape, wl.seq_len, wl.shape.d_model
+    hid, off = torch.zeros(seq, d, dtype=torch.bfloat16, device="cuda"), torch.full((2,), -1, dtype=torch.int32, device="cuda")
+    h0, mask, scores = pair.h0.cuda(), pair.mask.cuda(), inputs.make_scores(seq, 8).view(1, seq).cuda()
+    logits = torch.zeros(seq, shape.vocab, device="cuda")
+
+    def step():
+        pair.ctx.view("conf", 1, seq).copy_(scores)
+        hid.zero_(); logits.zero_(); off.fill_(-1)
+        pair.ctx.step(h0, mask, wl.k, 0.5, override_c=scores, hidden_out=hid, row_off=off, logits=logits)
+        state = [pair.ctx.view(name).clone() for name in ("kcache", "vcache", "conf", "pred", "c")]
+        return state + [hid.clone(), logits.clone(), off.clone()]
+
+    pair.gpu_step(10 ** 6, 1.0)
+    step()
+    want = step()
+    assert int(want[-1][1]) > wl.k
+    count = pair.ctx._view(pair.ctx.state.status + 128, 2, torch.int32)       # arrivals of the grid's CTAs, and of those that leave
+    assert count.tolist() == [0, 0]
+    count[0] = -2 ** 30
+    got = step()
+    assert count.tolist() == [0, 0]
+    with pytest.raises(binding.D2cError) as e:
+        pair.ctx.sync_status()
+    assert e.value.code == binding.D2C_ETIMEOUT and "site 60" in str(e.value)
+    assert got[-1].tolist() == [0, 0] and not got[-2].any() and not got[-3].any()
+    want_none = want[:2] + [scores] + want[3:5]                               # (of the step before; the confidences were put back since)
+    assert all(torch.equal(a, b) for a, b in zip(got[:5], want_none))
+    pair.ctx.view("status").zero_()
+    assert all(torch.equal(a, b) for a, b in zip(step(), want))
+    pair.ctx.sync_status()
+
+
 def test_an_older_error_of_the_caller_is_not_taken_for_a_launch_error():
     """The thread's last CUDA error may be the caller's own, of a call that has nothing to do with the library."""
     def older():                                                    # refused, and remembered as the last error
