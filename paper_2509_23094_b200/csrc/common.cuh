@@ -237,7 +237,7 @@ struct SmallArgs {
   bf16 *q, *o, *hmid; float* lse; float* abar; size_t abar_layer;
   float *c, *conf; int32_t* pred; CopyOut copies;
   int32_t* clear; int n_clear;                                   // words set to 0 on the way
-  int2* n_word; int n_tag;                                       // optional host words: the row count, and which step wrote it
+  uint64_t* n_word; int n_tag;                                   // optional host word: the row count and, in its upper half, which step wrote it
   uint32_t* sync; int32_t* status;                               // two counters that are zero between launches
   float4* lm_stats; float* rp;   // scratch, see small_step_scratch
 };

@@ -547,7 +547,7 @@ static int step_in_one_launch(d2c_ctx* ctx, const d2c_step_args* a, const d2c_st
   s.layer_in = out ? static_cast<bf16*>(out->layer_in) : nullptr; s.rows_cap = R;
   s.logits = out ? out->logits : nullptr;
   s.copies = index_outputs(ctx, out, R, B);
-  if (track) { s.n_word = reinterpret_cast<int2*>(ctx->hint_dev[slot]); s.n_tag = (int)ctx->step_no; }
+  if (track) { s.n_word = reinterpret_cast<uint64_t*>(ctx->hint_dev[slot]); s.n_tag = (int)ctx->step_no; }
   small_step_scratch(s, ctx->small_clusters, b.sk_partials, &s);
   D2C_TRY(ctx, launch_small_step(s, ctx->small_clusters, ctx->stream));
   if (track) { ctx->hint_step[slot] = ctx->step_no; ctx->hint_tagged[slot] = true; }

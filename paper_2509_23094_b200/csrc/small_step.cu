@@ -214,7 +214,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
     if (lane == 0) s_off[0] = s_lmoff[0] = s_toff[0] = 0;
     const int total = __shfl_sync(0xffffffffu, st, B - 1);
     if (lane <= ncl) s_ct[lane] = quot(lane * total, ncl);     // first tile of each cluster
-    if (lane == B - 1 && blockIdx.x == 0 && a.n_word) asm volatile("st.volatile.global.v2.u32 [%0], {%1, %2};" ::"l"(a.n_word), "r"(sn), "r"(a.n_tag) : "memory");
+    if (lane == B - 1 && blockIdx.x == 0 && a.n_word)
+      // (64 bits at once: of a vector store the host may see one half before the other)
+      asm volatile("st.relaxed.sys.global.u64 [%0], %1;" ::"l"(a.n_word), "l"((unsigned long long)(uint32_t)a.n_tag << 32 | (uint32_t)sn) : "memory");
   }
   __syncthreads();
   const int t0 = s_ct[cidx], mt = min(s_ct[cidx + 1] - t0, MAXT);
