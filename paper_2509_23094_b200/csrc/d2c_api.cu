@@ -162,6 +162,7 @@ struct d2c_ctx {
   long long hint_step[2] = {-1, -1};     // step number whose count the word holds
   bool hint_tagged[2] = {false, false};  // it was a step in one launch: it writes its number behind the count, in one store
   long long step_no = 0;
+  int asked_k = 0; float asked_p = 0.f;  // rows of stage 1 at most, and mass of stage 2, that the step before asked for
   bool few_rows = false;                 // this step's regime: at most 128 rows expected
   std::vector<MapCache> maps;            // six launches of each layer (QKV, forward, probabilities, output, gate/up, down), LM head
   int max_pairs = 0;                     // SM pairs the projections of this step may use (0: all)
@@ -535,6 +536,13 @@ static bool few_for_one_launch(const d2c_ctx* ctx, int batch, int room, int rows
   const int most = c.d_model > 256 || (long long)c.vocab * c.d_model > 1 << 18 ? 1 : 2 * rows <= room ? 3 : 2;
   return batch * ceil_div(rows, 16 * batch) <= ctx->small_clusters * most;
 }
+// Rows that stage 1 of a call selects at most.
+static int most_of_stage1(const d2c_step_args* a) {
+  const int lo = a->block_lo > 0 ? a->block_lo : 0, hi = a->block_hi < a->seq_len ? a->block_hi : a->seq_len;
+  const int width = a->block_hi > a->block_lo ? (hi > lo ? hi - lo : 0) : a->seq_len;
+  return a->k < width ? a->k : width;
+}
+static void note_asked(d2c_ctx* ctx, const d2c_step_args* a) { ctx->asked_k = most_of_stage1(a); ctx->asked_p = a->p; }
 // It is on the caller's stream.
 static int step_in_one_launch(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out, bool track) {
   const d2c_config& c = ctx->cfg;
@@ -551,7 +559,7 @@ static int step_in_one_launch(d2c_ctx* ctx, const d2c_step_args* a, const d2c_st
   small_step_scratch(s, ctx->small_clusters, b.sk_partials, &s);
   D2C_TRY(ctx, launch_small_step(s, ctx->small_clusters, ctx->stream));
   if (track) { ctx->hint_step[slot] = ctx->step_no; ctx->hint_tagged[slot] = true; }
-  ctx->step_no++;
+  ctx->step_no++; note_asked(ctx, a);
   if (ctx->early_hidden_host && ctx->copy_stream) {           // d2c_step_host's rows
     if (ctx->early_hidden_dev) { D2C_TRY(ctx, launch_rows_to_host(s.x, b.row_off + B, c.d_model, ctx->early_hidden_dev, ctx->stream)); }
     else D2C_TRY(ctx, cu(cudaMemcpyAsync(ctx->early_hidden_host, s.x, (size_t)R * c.d_model * sizeof(bf16), cudaMemcpyDeviceToHost, ctx->stream)));
@@ -569,12 +577,17 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
       return fail(ctx, D2C_EINVAL, "d2c_step: h0 and hidden_out must be 16-byte aligned");
   }
   if (ctx->small_clusters > 0 && !ctx->prof && !(out && reinterpret_cast<uintptr_t>(out->layer_in) % 16)) {
-    // One launch where few rows are expected, going by the step before like everything here, or where there is room for no more.
+    // One launch where few rows are expected, going by the step before like everything here, or where there is room for no more.  Not where
+    // the call asks for more than that one did, so that its count says nothing: many rows behind few cost the separate kernels hardly
+    // more than behind many, and the one launch several passes a cluster.  Behind 16 + 2 % of the rows, us, separate / one launch, all rows of
+    // one layer of d 256: 600 positions 79 / 105, 2048 155 / 376, 4096 390 / 1011; three layers, four of 700 248 / 746; three of d 512, 2048 528 / 1516;
+    // 16 + 90 %: 143 / 250 at 2048, 343 / 703 at 4096.
     const int rows = a->batch * a->seq_len;
     const bool capturing = stream_captures(ctx), any = few_for_one_launch(ctx, a->batch, rows, rows);
     const bool track = ctx->hint_host[0] != nullptr && !capturing && (!any || ctx->host_call);
     int expect = rows;
-    if (!any) D2C_TRY(ctx, previous_rows(ctx, capturing, &expect));
+    const bool asks_more = most_of_stage1(a) > ctx->asked_k || a->p > ctx->asked_p;
+    if (!any && !asks_more) D2C_TRY(ctx, previous_rows(ctx, capturing, &expect));
     if (few_for_one_launch(ctx, a->batch, rows, expect)) return step_in_one_launch(ctx, a, out, track);
   }
   // critical path on `st`, probabilities + rollout on `side` (the same stream while profiling or when serial)
@@ -660,7 +673,7 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     D2C_TRY(ctx, cu(cudaEventRecord(ctx->ev_hint[slot], st)));
     ctx->hint_step[slot] = ctx->step_no; ctx->hint_tagged[slot] = false;
   }
-  ctx->step_no++;
+  ctx->step_no++; note_asked(ctx, a);
   const int32_t* n_rows = b.row_off + B;
   const int32_t* n_lm = b.lm_off + B;
 

@@ -1,0 +1,99 @@
+"""Which kernels a step is made of, without a device: the library runs over a CUDA runtime that does nothing but note the launches
+(tests/host/fake_cudart.c).  The row counts that steps leave for the host are written by the test, as the kernels would.  Each test is a
+process of its own, as the library takes the runtime that it finds first."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+from paper_2509_23094_b200 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes as C, sys, types
+from dataclasses import replace
+sys.modules["torch"] = types.ModuleType("torch")          # (only names of it are in annotations)
+sys.path.insert(0, sys.argv[1])
+from paper_2509_23094_b200 import binding, inputs
+lib, fake = binding.load(), C.CDLL("libcudart.so.12")
+fake.fake_log.restype = C.c_char_p
+fake.fake_host_words.restype = C.POINTER(C.c_int32)
+fake.fake_refuse.argtypes = [C.c_char_p, C.c_int]
+
+
+class Ctx:
+    def __init__(self, shape, batch, seq, flags=0):
+        cfg = binding.make_config(shape, batch, seq, flags=flags)
+        self.batch, self.seq, self.n = batch, seq, 0
+        w, at = binding.Weights(), (C.c_void_p * shape.n_layers)(*[1 << 20] * shape.n_layers)
+        for name in ("wqkv", "bqkv", "wo", "w_gate", "w_up", "w_down", "g_attn", "g_ffn"):
+            setattr(w, name, C.cast(at, C.POINTER(C.c_void_p)))
+        w.g_final = w.w_lm = 1 << 20
+        self.handle = C.c_void_p()
+        need = lib.d2c_workspace_bytes(C.byref(cfg))
+        binding._check(lib.d2c_create(C.byref(cfg), C.byref(w), 1 << 30, need, None, C.byref(self.handle)))
+        self.words = fake.fake_host_words()
+
+    def step(self, k, p, rows, block=(0, 0)):
+        # the kernels of a step that then finds `rows` rows
+        fake.fake_clear()
+        a = binding.StepArgs(self.batch, self.seq, 1 << 21, 1 << 22, None, None, k, p, None, None, *block)
+        rc = lib.d2c_step(self.handle, C.byref(a), None)
+        slot = 2 * (self.n & 1)
+        self.words[slot], self.words[slot + 1] = rows, self.n
+        self.n += 1
+        if rc:
+            return rc
+        names = fake.fake_log().decode().split()
+        assert names
+        one = [n for n in names if "small_step_kernel" in n]
+        assert not one or len(names) == 1
+        return "one" if one else "separate"
+"""
+
+
+@pytest.fixture(scope="module")
+def runtime(tmp_path_factory):
+    build.build()
+    d = tmp_path_factory.mktemp("fake_cuda")
+    (d / "v.map").write_text("libcudart.so.12 { *; };\n")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-Wall", "-Werror", "-o", str(d / "libcudart.so.12"), os.path.join(HERE, "host", "fake_cudart.c"),
+                    "-Wl,-soname,libcudart.so.12", f"-Wl,--version-script={d / 'v.map'}"], check=True)
+    return str(d)
+
+
+def _run(runtime, body):
+    r = subprocess.run([sys.executable, "-c", PRELUDE + textwrap.dedent(body), ROOT], env=dict(os.environ, LD_LIBRARY_PATH=runtime),
+                       stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout
+
+
+def test_small_steps_go_by_the_count_of_a_step_that_asked_for_no_less(runtime):
+    """Few rows behind few of the same call: one launch.  A call that asks for more rows of stage 1 or for more of the mass than the step
+    before did, as the select-all step of the next request does, takes the separate kernels, whatever that one found."""
+    _run(runtime, """
+    c = Ctx(inputs.TOY, 1, 2048)
+    few = (16, 0.1, 40)
+    assert c.step(2048, 1.0, 2048) == "separate"
+    assert c.step(*few) == "separate"                                    # behind many
+    assert c.step(*few) == "one" and c.step(*few) == "one"
+    for more in ((2048, 1.0), (16, 0.9), (17, 0.1), (10 ** 6, 0.1)):
+        assert c.step(*more, 2048) == "separate", more
+        assert c.step(*few) == "separate"                                # behind many
+        assert c.step(*few) == "one"
+    assert c.step(8, 0.05, 20) == "one" and c.step(16, 0.05, 30) == "separate" and c.step(16, 0.05, 30) == "one"
+    assert c.step(16, 0.0, 2000) == "one" and c.step(16, 0.0, 16) == "separate" and c.step(16, 0.0, 16) == "one"      # (found many: the next goes by it)
+    assert c.step(2048, 0.0, 32, block=(100, 132)) == "separate"          # of a block 32 at most, more than 16
+    assert c.step(2048, 0.0, 32, block=(132, 164)) == "one" and c.step(2048, 0.0, 32, block=(0, 32)) == "one"
+    assert c.step(2048, 0.0, 32, block=(2040, 4096)) == "one"             # eight positions of it are there
+    assert c.step(2048, 0.0, 32, block=(164, 196)) == "separate"
+    assert c.step(2048, 0.0, 500) == "separate"
+    c = Ctx(inputs.TOY, 1, 128)                                            # room for few rows only
+    assert c.step(128, 1.0, 128) == "one" and c.step(8, 0.5, 60) == "one" and c.step(128, 1.0, 128) == "one"
+    c = Ctx(inputs.TOY, 1, 2048, flags=16)                                 # a flag that asks for the separate kernels
+    assert all(c.step(*few) == "separate" for _ in range(4))
+    """)
