@@ -576,6 +576,10 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     if (reinterpret_cast<uintptr_t>(x) % 16 || reinterpret_cast<uintptr_t>(a->h0) % 16)
       return fail(ctx, D2C_EINVAL, "d2c_step: h0 and hidden_out must be 16-byte aligned");
   }
+  // the row count of the previous step, read behind that step's selection, once (a call for an event or the stream takes 0.5 us)
+  const bool capturing = stream_captures(ctx);
+  int expect_rows = 1 << 30;
+  bool read = false;
   if (ctx->small_clusters > 0 && !ctx->prof && !(out && reinterpret_cast<uintptr_t>(out->layer_in) % 16)) {
     // One launch where few rows are expected, going by the step before like everything here, or where there is room for no more.  Not where
     // the call asks for more than that one did, so that its count says nothing: many rows behind few cost the separate kernels hardly
@@ -583,12 +587,11 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     // one layer of d 256: 600 positions 79 / 105, 2048 155 / 376, 4096 390 / 1011; three layers, four of 700 248 / 746; three of d 512, 2048 528 / 1516;
     // 16 + 90 %: 143 / 250 at 2048, 343 / 703 at 4096.
     const int rows = a->batch * a->seq_len;
-    const bool capturing = stream_captures(ctx), any = few_for_one_launch(ctx, a->batch, rows, rows);
+    const bool any = few_for_one_launch(ctx, a->batch, rows, rows);
     const bool track = ctx->hint_host[0] != nullptr && !capturing && (!any || ctx->host_call);
-    int expect = rows;
     const bool asks_more = most_of_stage1(a) > ctx->asked_k || a->p > ctx->asked_p;
-    if (!any && !asks_more) D2C_TRY(ctx, previous_rows(ctx, capturing, &expect));
-    if (few_for_one_launch(ctx, a->batch, rows, expect)) return step_in_one_launch(ctx, a, out, track);
+    if (!any) { D2C_TRY(ctx, previous_rows(ctx, capturing, &expect_rows)); read = true; }
+    if (few_for_one_launch(ctx, a->batch, rows, any || asks_more || expect_rows > rows ? rows : expect_rows)) return step_in_one_launch(ctx, a, out, track);
   }
   // critical path on `st`, probabilities + rollout on `side` (the same stream while profiling or when serial)
   const int B = a->batch, L = a->seq_len, R = B * L, d = c.d_model;
@@ -622,11 +625,10 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
   // with few rows or in small models, for a single layer whose products leave SMs free (it then overlaps the LM head), and on SM
   // pairs that the projections leave alone.  Otherwise a statically scheduled GEMM whose CTAs start late behind side-stream CTAs
   // loses more than the overlap gains (measured at 488 rows x 32 layers: +5 %).
-  // regime of this step: the row count of the previous step, read behind that step's selection kernel
-  const bool capturing = stream_captures(ctx), track = ctx->hint_host[0] != nullptr && !capturing;
+  // regime of this step: the row count of the previous step
+  const bool track = ctx->hint_host[0] != nullptr && !capturing;
   const int slot = (int)(ctx->step_no & 1);
-  int expect_rows = 1 << 30;
-  D2C_TRY(ctx, previous_rows(ctx, capturing, &expect_rows));
+  if (!read) D2C_TRY(ctx, previous_rows(ctx, capturing, &expect_rows));
   ctx->few_rows = expect_rows <= 128;
   const bool few_rows = ctx->few_rows;
   // With few rows the projections stream weights and 96 of the 148 SMs take all the HBM gives (32 layers at 81 rows: 64

@@ -17,12 +17,13 @@ static size_t log_len;
 static const char* refuse_name = "";             /* launches of kernels whose name has this in it ... */
 static err refuse_with;                          /* ... return this */
 static void* host_words;                         /* the last mapped host memory handed out */
-static int capturing;
+static int capturing, asked;                     /* asked: of an event or of a stream's state */
 const char* fake_log(void) { return log_; }
 void fake_clear(void) { log_len = 0; log_[0] = 0; }
 void fake_refuse(const char* name, int with) { refuse_name = strdup(name); refuse_with = with; }
 void* fake_host_words(void) { return host_words; }
 void fake_capture(int on) { capturing = on; }
+int fake_asked(void) { const int n = asked; asked = 0; return n; }
 
 /* ---- registration and launches ---- */
 static struct { const void* fun; const char* name; } kernels[4096];
@@ -58,7 +59,7 @@ err cudaEventCreateWithFlags(void** e, unsigned f) { (void)f; *e = malloc(1); re
 err cudaEventDestroy(void* e) { free(e); return 0; }
 err cudaEventElapsedTime(float* ms, void* a, void* b) { (void)a; (void)b; *ms = 0; return 0; }
 err cudaEventRecord(void* e, void* s) { (void)e; (void)s; return 0; }
-err cudaEventSynchronize(void* e) { (void)e; return 0; }
+err cudaEventSynchronize(void* e) { (void)e; ++asked; return 0; }
 err cudaHostAlloc(void** p, size_t n, unsigned f) { (void)f; host_words = *p = calloc(1, n); return 0; }
 err cudaFreeHost(void* p) { free(p); return 0; }
 err cudaHostGetDevicePointer(void** d, void* h, unsigned f) { (void)f; *d = h; return 0; }
@@ -81,7 +82,7 @@ err cudaPointerGetAttributes(void* a, const void* p) { (void)a; (void)p; last = 
 err cudaStreamCreateWithFlags(void** s, unsigned f) { (void)f; *s = malloc(1); return 0; }
 err cudaStreamCreateWithPriority(void** s, unsigned f, int p) { (void)f; (void)p; *s = malloc(1); return 0; }
 err cudaStreamDestroy(void* s) { free(s); return 0; }
-err cudaStreamIsCapturing(void* s, int* v) { (void)s; *v = capturing; return 0; }
-err cudaStreamQuery(void* s) { (void)s; return 0; }
+err cudaStreamIsCapturing(void* s, int* v) { (void)s; *v = capturing; ++asked; return 0; }
+err cudaStreamQuery(void* s) { (void)s; ++asked; return 0; }
 err cudaStreamSynchronize(void* s) { (void)s; return 0; }
 err cudaStreamWaitEvent(void* s, void* e, unsigned f) { (void)s; (void)e; (void)f; return 0; }

@@ -97,3 +97,19 @@ def test_small_steps_go_by_the_count_of_a_step_that_asked_for_no_less(runtime):
     c = Ctx(inputs.TOY, 1, 2048, flags=16)                                 # a flag that asks for the separate kernels
     assert all(c.step(*few) == "separate" for _ in range(4))
     """)
+
+
+def test_a_step_asks_once_for_the_count_of_the_one_before(runtime):
+    """Whether the stream is captured, and the event behind the selection of the step before: each a call of 0.5 us in front of the step's
+    first launch, made once whichever way the step then goes."""
+    _run(runtime, """
+    for shape in (inputs.TOY, inputs.TOY_HD128):
+        c = Ctx(shape, 1, 2048)
+        for i in range(4):
+            assert c.step(2048, 1.0, 2048) == "separate"
+            assert fake.fake_asked() == 2, (shape.name, i)
+    c = Ctx(inputs.TOY, 1, 2048)
+    assert [c.step(16, 0.1, 40) for _ in range(3)] == ["separate", "one", "one"]
+    fake.fake_asked()
+    assert c.step(16, 0.1, 40) == "one" and fake.fake_asked() == 1           # (the count of a step in one launch is behind no event)
+    """)
