@@ -834,28 +834,23 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
   }
 }
 
-int config(int clusters, cudaStream_t st, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
-  static PerDevice attr_set;
-  if (attr_set.first()) {
-    D2C_CUDA_OK(cudaFuncSetAttribute(small_step_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    D2C_CUDA_OK(cudaFuncSetAttribute(small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem));
-  }
+void config(int clusters, cudaStream_t st, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   cfg->gridDim = dim3(clusters * CL); cfg->blockDim = dim3(NT); cfg->dynamicSmemBytes = kSmallSmem; cfg->stream = st;
   attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
   cfg->attrs = attr; cfg->numAttrs = 1;
-  return D2C_OK;
 }
 }  // namespace
 
+// Asked for by every context when it is made, which sets the attributes that its launches need: kept from the first time on, one thread
+// would find them done that another is only about to set, and take the refusal for the answer.
 int small_step_clusters() {
-  static int known[kMaxDevices] = {};                          // looked up once per device, +1
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-  if (known[dev]) return known[dev] - 1;
+  int n = 0;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  if (config(1, nullptr, &cfg, attr) != D2C_OK || cudaOccupancyMaxActiveClusters(&n, small_step_kernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
-  known[dev] = n + 1;
+  config(1, nullptr, &cfg, attr);
+  if (cudaFuncSetAttribute(small_step_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute(small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, small_step_kernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
   return n;
 }
 
@@ -872,8 +867,7 @@ size_t small_step_scratch(const SmallArgs& a, int clusters, float* base, SmallAr
 int launch_small_step(const SmallArgs& a, int clusters, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  const int rc = config(clusters, st, &cfg, attr);
-  if (rc != D2C_OK) return rc;
+  config(clusters, st, &cfg, attr);
   D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, small_step_kernel, a));
   count_launch(1);
   return D2C_OK;

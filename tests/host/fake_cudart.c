@@ -16,11 +16,13 @@ static char log_[1 << 20];
 static size_t log_len;
 static const char* refuse_name = "";             /* launches of kernels whose name has this in it ... */
 static err refuse_with;                          /* ... return this */
+static int unset;                                /* so many calls that set an attribute fail */
 static void* host_words;                         /* the last mapped host memory handed out */
 static int capturing, asked;                     /* asked: of an event or of a stream's state */
 const char* fake_log(void) { return log_; }
 void fake_clear(void) { log_len = 0; log_[0] = 0; }
 void fake_refuse(const char* name, int with) { refuse_name = strdup(name); refuse_with = with; }
+void fake_unset(int calls) { unset = calls; }
 void* fake_host_words(void) { return host_words; }
 void fake_capture(int on) { capturing = on; }
 int fake_asked(void) { const int n = asked; asked = 0; return n; }
@@ -63,7 +65,7 @@ err cudaEventSynchronize(void* e) { (void)e; ++asked; return 0; }
 err cudaHostAlloc(void** p, size_t n, unsigned f) { (void)f; host_words = *p = calloc(1, n); return 0; }
 err cudaFreeHost(void* p) { free(p); return 0; }
 err cudaHostGetDevicePointer(void** d, void* h, unsigned f) { (void)f; *d = h; return 0; }
-err cudaFuncSetAttribute(const void* f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
+err cudaFuncSetAttribute(const void* f, int a, int v) { (void)f; (void)a; (void)v; if (unset > 0) { --unset; return last = 1; } return 0; }
 static err encode(void) { return 0; }
 err cudaGetDriverEntryPoint(const char* name, void** fn, unsigned long long flags, int* found) {
   (void)flags;

@@ -113,3 +113,15 @@ def test_a_step_asks_once_for_the_count_of_the_one_before(runtime):
     fake.fake_asked()
     assert c.step(16, 0.1, 40) == "one" and fake.fake_asked() == 1           # (the count of a step in one launch is behind no event)
     """)
+
+
+def test_a_context_counts_clusters_for_itself(runtime):
+    """What the first context of a process found while its kernel's attributes could not be set, or were not set yet by the thread that had
+    begun to, is not what the others find."""
+    _run(runtime, """
+    fake.fake_unset(1)
+    a = Ctx(inputs.TOY, 1, 128)
+    fake.fake_unset(0)
+    b = Ctx(inputs.TOY, 1, 128)
+    assert a.step(128, 1.0, 128) == "separate" and b.step(128, 1.0, 128) == "one"
+    """)
