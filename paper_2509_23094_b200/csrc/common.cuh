@@ -244,7 +244,7 @@ struct SmallArgs {
 int small_step_clusters();                                       // clusters that fit the GPU together (0: none)
 // Places the scratch of a launch from `base` on (null out: only its size); floats.
 size_t small_step_scratch(const SmallArgs& a, int clusters, float* base, SmallArgs* out);
-int launch_small_step(const SmallArgs& a, int clusters, cudaStream_t st);
+int launch_small_step(const SmallArgs& a, int clusters, cudaStream_t st, bool* refused);       // refused: there is no room for it, nothing is enqueued
 
 }  // namespace d2c
 

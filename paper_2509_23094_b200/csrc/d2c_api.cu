@@ -543,8 +543,9 @@ static int most_of_stage1(const d2c_step_args* a) {
   return a->k < width ? a->k : width;
 }
 static void note_asked(d2c_ctx* ctx, const d2c_step_args* a) { ctx->asked_k = most_of_stage1(a); ctx->asked_p = a->p; }
-// It is on the caller's stream.
-static int step_in_one_launch(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out, bool track) {
+// It is on the caller's stream.  Where the GPU has no room for it, as in a part of one that has fewer SMs than were counted, the context goes
+// on with the separate kernels.
+static int step_in_one_launch(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out, bool track, bool* refused) {
   const d2c_config& c = ctx->cfg;
   const Buffers& b = ctx->buf;
   const int B = a->batch, L = a->seq_len, R = B * L, slot = (int)(ctx->step_no & 1);
@@ -557,7 +558,8 @@ static int step_in_one_launch(d2c_ctx* ctx, const d2c_step_args* a, const d2c_st
   s.copies = index_outputs(ctx, out, R, B);
   if (track) { s.n_word = reinterpret_cast<uint64_t*>(ctx->hint_dev[slot]); s.n_tag = (int)ctx->step_no; }
   small_step_scratch(s, ctx->small_clusters, b.sk_partials, &s);
-  D2C_TRY(ctx, launch_small_step(s, ctx->small_clusters, ctx->stream));
+  D2C_TRY(ctx, launch_small_step(s, ctx->small_clusters, ctx->stream, refused));
+  if (*refused) { ctx->small_clusters = 0; return D2C_OK; }
   if (track) { ctx->hint_step[slot] = ctx->step_no; ctx->hint_tagged[slot] = true; }
   ctx->step_no++; note_asked(ctx, a);
   if (ctx->early_hidden_host && ctx->copy_stream) {           // d2c_step_host's rows
@@ -591,7 +593,11 @@ int d2c_step(d2c_ctx* ctx, const d2c_step_args* a, const d2c_step_out* out) {
     const bool track = ctx->hint_host[0] != nullptr && !capturing && (!any || ctx->host_call);
     const bool asks_more = most_of_stage1(a) > ctx->asked_k || a->p > ctx->asked_p;
     if (!any) { D2C_TRY(ctx, previous_rows(ctx, capturing, &expect_rows)); read = true; }
-    if (few_for_one_launch(ctx, a->batch, rows, any || asks_more || expect_rows > rows ? rows : expect_rows)) return step_in_one_launch(ctx, a, out, track);
+    if (few_for_one_launch(ctx, a->batch, rows, any || asks_more || expect_rows > rows ? rows : expect_rows)) {
+      bool refused = false;
+      const int rc = step_in_one_launch(ctx, a, out, track, &refused);
+      if (!refused) return rc;
+    }
   }
   // critical path on `st`, probabilities + rollout on `side` (the same stream while profiling or when serial)
   const int B = a->batch, L = a->seq_len, R = B * L, d = c.d_model;

@@ -864,11 +864,15 @@ size_t small_step_scratch(const SmallArgs& a, int clusters, float* base, SmallAr
   return at;
 }
 
-int launch_small_step(const SmallArgs& a, int clusters, cudaStream_t st) {
+int launch_small_step(const SmallArgs& a, int clusters, cudaStream_t st, bool* refused) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   config(clusters, st, &cfg, attr);
-  D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, small_step_kernel, a));
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, small_step_kernel, a);
+  // (what says that so many clusters do not fit here together, and nothing about the work before)
+  *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported;
+  if (*refused) { (void)cudaGetLastError(); return D2C_OK; }
+  D2C_CUDA_OK(e);
   count_launch(1);
   return D2C_OK;
 }

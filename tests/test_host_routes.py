@@ -125,3 +125,24 @@ def test_a_context_counts_clusters_for_itself(runtime):
     b = Ctx(inputs.TOY, 1, 128)
     assert a.step(128, 1.0, 128) == "separate" and b.step(128, 1.0, 128) == "one"
     """)
+
+
+# cudaErrorInvalidValue, cudaErrorLaunchOutOfResources, cudaErrorIllegalAddress, cudaErrorCooperativeLaunchTooLarge, cudaErrorInvalidClusterSize
+@pytest.mark.parametrize("code,goes_on", [(1, False), (701, True), (700, False), (720, True), (912, True)])
+def test_a_refused_one_launch_step_takes_the_separate_kernels(runtime, code, goes_on):
+    """A GPU that has fewer SMs than were counted (a part of one) refuses a launch that needs all its CTAs at once: the step is done by the
+    separate kernels, and so are those behind it.  Any other error is the call's answer, and nothing else is enqueued."""
+    _run(runtime, f"""
+    c = Ctx(inputs.TOY, 1, 128)
+    assert c.step(128, 1.0, 128) == "one"
+    fake.fake_refuse(b"small_step_kernel", {code})
+    if {goes_on}:
+        assert c.step(8, 0.5, 60) == "separate" and fake.cudaGetLastError() == 0
+        fake.fake_refuse(b"", 0)
+        assert c.step(8, 0.5, 60) == "separate"
+    else:
+        assert c.step(8, 0.5, 60) == binding.D2C_ECUDA and fake.fake_log() == b""
+        c.n -= 1                                                           # (a step that was not enqueued)
+        fake.fake_refuse(b"", 0)
+        assert c.step(8, 0.5, 60) == "one"
+    """)
