@@ -906,7 +906,7 @@ attn_abar_tc(const __grid_constant__ AbarMaps maps, const AttnTcParams p) {
 
 // True if the tcgen05 kernels can take this problem (otherwise the caller uses the mma.sync ones).
 bool attention_tc_supported(const AttnArgs& a) {
-  return a.dh == ADH && a.hq <= 512 && a.hq / a.hkv <= AQ && a.q_rows >= AQ && (long long)a.batch * a.cache_seq >= AKEYS && (a.ldq & 7) == 0 &&
+  return a.dh == ADH && a.hq <= 512 && a.q_rows >= AQ && (long long)a.batch * a.cache_seq >= AKEYS && (a.ldq & 7) == 0 &&
          (reinterpret_cast<uintptr_t>(a.q) & 15) == 0 && (reinterpret_cast<uintptr_t>(a.kc) & 15) == 0 &&
          (reinterpret_cast<uintptr_t>(a.vc) & 15) == 0;
 }
@@ -1018,7 +1018,7 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     return splits;
   };
   const int solo = splits_of(ceil_div(rows_seq, AQ) * a.hq * a.batch), packed = AQ / (a.hq / a.hkv);
-  const bool pack = solo == 1 || solo < splits_of(ceil_div(rows_seq, packed) * a.hkv * a.batch);
+  const bool pack = packed > 0 && (solo == 1 || solo < splits_of(ceil_div(rows_seq, packed) * a.hkv * a.batch));      // (a tile has no place for more than 128 heads)
   const int group = pack ? a.hq / a.hkv : 1, heads = a.hq / group, tile_rows = AQ / group;
   AttnTcParams p{a, status, sms, 1, 1, 128, 0, group, heads, a.hq / a.hkv / group, tile_rows, 0, 0};
   if (a.which != 2) {

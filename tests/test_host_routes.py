@@ -146,3 +146,14 @@ def test_a_refused_one_launch_step_takes_the_separate_kernels(runtime, code, goe
         fake.fake_refuse(b"", 0)
         assert c.step(8, 0.5, 60) == "one"
     """)
+
+
+def test_attention_of_more_query_heads_than_a_tile_has_rows(runtime):
+    """129 query heads and more of a K/V head do not share a tile of 128 rows; each then has tiles of its own, on the tensor cores like any."""
+    _run(runtime, """
+    for heads in (128, 129, 160, 512):
+        c = Ctx(replace(inputs.TOY_HD128, name="many", n_layers=1, n_q_heads=heads, n_kv_heads=1), 1, 300)
+        for rows in (300, 20, 20):
+            assert c.step(16, 0.1, rows) == "separate"
+            assert "attn_fwd_tc" in fake.fake_log().decode(), (heads, rows)
+    """)
