@@ -1050,6 +1050,7 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     // 3810 -> 3775 us against one for each, but two of d 512, all of 521 rows, 128 -> 134)
     const int most = heads * a.batch * ((xtiles + 1) / 2), single = heads * a.batch * xtiles < sms ? heads * a.batch * xtiles : sms;
     const int clusters = 2 * ceil_div(rows_seq, tile_rows) > xtiles ? xtiles : (xtiles + 1) / 2;
+    if ((long long)clusters * a.batch > 65535) p.splits = 1;      // (tiles of a few rows, of many long sequences: the grid has no room for their places)
     const int pairs = ceil_div(ceil_div(rows_seq, tile_rows), 2) * heads * a.batch;      // (expected; where none are to be split, looking for them costs 0.4 us)
     p.split_last = units > sms && pairs > sms && pairs % sms > 0 && 2 * (pairs % sms) <= sms;
     // By place where all places run at once: two layers of d 512, all rows of eight sequences of 300, 179.7 -> 177.8 us a step.

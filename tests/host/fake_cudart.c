@@ -40,15 +40,16 @@ void __cudaRegisterFunction(void** h, const char* fun, char* dev, const char* na
 void __cudaRegisterVar(void** h, char* v, char* d, const char* n, int a, size_t s, int b, int c) { (void)h; (void)v; (void)d; (void)n; (void)a; (void)s; (void)b; (void)c; }
 err __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* s, void* st) { (void)g; (void)b; (void)s; (void)st; return 1; }
 static err last;
-static err launch(const void* fun) {
+static err launch(const void* fun, dim3 grid) {
+  if (!grid.x || !grid.y || !grid.z || grid.x > 0x7fffffffu || grid.y > 65535 || grid.z > 65535) return last = 9;      /* cudaErrorInvalidConfiguration */
   const char* name = "?";
   for (int i = 0; i < n_kernels; ++i) if (kernels[i].fun == fun) name = kernels[i].name;
   if (refuse_with && *refuse_name && strstr(name, refuse_name)) { last = refuse_with; return refuse_with; }
   if (log_len + strlen(name) + 2 < sizeof(log_)) log_len += (size_t)sprintf(log_ + log_len, "%s\n", name);
   return 0;
 }
-err cudaLaunchKernelExC(const launch_config* c, const void* fun, void** args) { (void)c; (void)args; return launch(fun); }
-err cudaLaunchKernel(const void* fun, dim3 g, dim3 b, void** args, size_t s, void* st) { (void)g; (void)b; (void)args; (void)s; (void)st; return launch(fun); }
+err cudaLaunchKernelExC(const launch_config* c, const void* fun, void** args) { (void)args; return launch(fun, c->grid); }
+err cudaLaunchKernel(const void* fun, dim3 g, dim3 b, void** args, size_t s, void* st) { (void)b; (void)args; (void)s; (void)st; return launch(fun, g); }
 
 /* ---- the rest ---- */
 err cudaGetLastError(void) { const err e = last; last = 0; return e; }

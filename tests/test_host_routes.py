@@ -157,3 +157,13 @@ def test_attention_of_more_query_heads_than_a_tile_has_rows(runtime):
             assert c.step(16, 0.1, rows) == "separate"
             assert "attn_fwd_tc" in fake.fake_log().decode(), (heads, rows)
     """)
+
+
+def test_attention_of_few_rows_of_many_long_sequences(runtime):
+    """Tiles of a few rows, room for thousands of them in each of many sequences: no dimension of a grid has room for all of them."""
+    _run(runtime, """
+    for heads, batch in ((32, 64), (32, 66), (128, 16), (64, 32)):
+        c = Ctx(replace(inputs.TOY_HD128, name="long", n_layers=1, n_q_heads=heads, n_kv_heads=1), batch, 8192)
+        for rows in (8192 * batch, batch, batch, 2 * batch, 4 * batch, 40 * batch):
+            assert c.step(1, 0.1, rows) == "separate", (heads, batch, rows, lib.d2c_last_error(c.handle))
+    """)
