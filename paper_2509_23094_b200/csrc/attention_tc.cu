@@ -1090,9 +1090,12 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     if (rc != D2C_OK) { if (a.cache[1]) a.cache[1]->forget(); return rc; }
   }
   cudaLaunchConfig_t cfg = {};
-  // Where there is room for twice as many tiles of rows as are expected, or more, the live items are numbered in turn, as in the forward:
-  // 300 rows of five sequences x 3071 keys 100.5 -> 95.8 us, 147 of four x 1187 32.4 -> 31.1, 420 of three x 1100 38.3 -> 37.8.  Finding its
-  // number takes a cluster up to 0.9 us, which it is not worth with fewer (260 of eight x 700 41.8 / 42.7) or one sequence.
+  // The live items are numbered in turn, as in the forward, where there is room for twice as many tiles of rows as are expected, or more, and
+  // so for more than two CTAs an SM that would find nothing to do.  us, by place / in turn: 300 rows of five sequences x 3071 keys 100.5 / 95.8,
+  // 147 of four x 1187 32.4 / 31.1, 420 of three x 1100 38.3 / 37.8.  Finding its number takes a cluster up to 0.9 us: with fewer tiles than that
+  // 260 rows of eight x 700 41.8 / 42.7.  Two to eight sequences of 300 to 2048 positions, 4 to 150 rows each, 4, 28 and 32 heads: with up to two
+  // empty CTAs an SM 1.5 more (8 rows of two x 701, 4 heads, 14.7 / 15.8) to 1.8 less (28 heads, 160 of eight x 701 20.0 / 18.1), beyond
+  // 0.3 to 9 less (28 heads, 32 rows of eight x 2048 36.5 / 30.5), but for 300 rows of two x 2048, 28.8 / 30.4.
   const int xs = 2 * p.head_groups * ceil_div(a.seq_len, 2 * AKEYS), worst_tiles = ceil_div(a.max_rows_per_seq, p.row_tile);
   const int empty = xs * a.batch * (worst_tiles - ceil_div(rows_seq, p.row_tile));
   const bool in_turn = a.batch > 1 && worst_tiles >= 2 * ceil_div(rows_seq, p.row_tile) && empty > 2 * sms;

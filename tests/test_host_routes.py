@@ -167,3 +167,18 @@ def test_attention_of_few_rows_of_many_long_sequences(runtime):
         for rows in (8192 * batch, batch, batch, 2 * batch, 4 * batch, 40 * batch):
             assert c.step(1, 0.1, rows) == "separate", (heads, batch, rows, lib.d2c_last_error(c.handle))
     """)
+
+
+def test_probabilities_of_few_rows_are_numbered_in_turn(runtime):
+    """The form of the probabilities kernel that the GPU test of it means to reach, with the rows that it has (p of the known ones)."""
+    from test_gpu_branches import IN_TURN
+    _run(runtime, f"""
+    for layers, batch, seq, heads, kv, p in {IN_TURN}:
+        c = Ctx(replace(inputs.TOY_HD128, name="turn", n_layers=layers, n_q_heads=heads, n_kv_heads=kv), batch, seq)
+        rows = batch * int(p * (seq - 100))
+        forms = []
+        for n in (batch * seq, rows, rows, rows):
+            c.step(0, p, n)
+            forms.append({{name.split("AbarFormE")[1][0] for name in fake.fake_log().decode().split() if "AbarForm" in name}})
+        assert forms == [{{"0"}}, {{"0"}}, {{"1"}}, {{"1"}}], (heads, seq, forms)
+    """)
