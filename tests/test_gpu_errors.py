@@ -200,6 +200,47 @@ def test_logits_that_are_not_numbers_reach_the_confidences(flags):
     assert bool(torch.isnan(conf3).all()) and bool((pred3 == 0x7fffffff).all())
 
 
+@pytest.mark.parametrize("vocab", [1024, 1018, 200])
+def test_logits_of_small_steps_that_are_not_numbers_or_infinite(vocab):
+    """The same of a small model, in one launch and in separate kernels: a feature that is not a number, hidden states that are not, one
+    that is infinite either way.  What is a number and the tokens are the same in each."""
+    shape, seq = replace(inputs.TOY, vocab=vocab), 112
+    wl = inputs.Workload("nan", shape, 1, seq, 40, 60, "random", 16, 0.2, seed=6)
+    w = inputs.make_weights(shape, seed=6, device="cuda")
+    mask = inputs.make_mask(wl)
+    h0, mask = torch.randn(1, seq, shape.d_model, generator=torch.Generator().manual_seed(3)), mask.cuda()
+    h0[0, :, 3] = 30.0 * (1 - 2 * (torch.arange(seq) % 2))           # (far more than a layer adds: the sign stays)
+    h0 = h0.to(torch.bfloat16).cuda()
+    at = mask[0].nonzero().flatten()
+    def run(w, h0, flags):
+        ctx = binding.Context(binding.make_config(shape, 1, seq, flags=flags), w)
+        ctx.step(h0, mask, seq, 1.0)
+        ctx.sync_status()
+        return ctx.view("conf", 1, seq)[0][at].clone(), ctx.view("pred", 1, seq)[0][at].clone()
+    kinds = (0, 16, 1 | 2)                                           # one launch, separate kernels, portable ones
+    good = [run(w, h0, f) for f in kinds]
+    unused = next(t for t in range(5, vocab) if not any(bool((pred == t).any()) for _, pred in good))
+    bad, inf = (dict(w, w_lm=w["w_lm"].clone()) for _ in range(2))
+    bad["w_lm"][unused] = float("nan")
+    inf["w_lm"][unused] = 0.0
+    inf["w_lm"][unused][3] = float("inf")                            # its logits are +inf or -inf by the sign of one element
+    nan_h0 = h0.clone()
+    nan_h0[:] = float("nan")
+    results = []
+    for f, (conf, pred) in zip(kinds, good):
+        assert bool(torch.isfinite(conf).all())
+        conf2, pred2 = run(bad, h0, f)
+        assert bool(torch.isnan(conf2).all()) and torch.equal(pred, pred2), f
+        conf3, pred3 = run(w, nan_h0, f)
+        assert bool(torch.isnan(conf3).all()) and bool((pred3 == 0x7fffffff).all()), f
+        results.append(run(inf, h0, f))
+    up = results[0][1] == unused
+    assert bool(up.any()) and bool((~up).any())
+    for conf, pred in results:
+        assert torch.equal(pred == unused, up) and torch.equal(torch.isnan(conf), up)
+        torch.testing.assert_close(conf[~up], results[2][0][~up], rtol=3e-2, atol=0)
+
+
 @pytest.mark.parametrize("rule", [0, 1, 2])
 def test_commit_passes_over_rows_that_predict_no_token(rule):
     """One sequence of two has hidden states that are not numbers: nothing of it is committed (its predictions are no rows of
