@@ -1053,10 +1053,13 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     if ((long long)clusters * a.batch > 65535) p.splits = 1;      // (tiles of a few rows, of many long sequences: the grid has no room for their places)
     const int pairs = ceil_div(ceil_div(rows_seq, tile_rows), 2) * heads * a.batch;      // (expected; where none are to be split, looking for them costs 0.4 us)
     p.split_last = units > sms && pairs > sms && pairs % sms > 0 && 2 * (pairs % sms) <= sms;
-    // By place where all places run at once: two layers of d 512, all rows of eight sequences of 300, 179.7 -> 177.8 us a step.
-    const bool by_place = p.splits == 1 && single < sms;
+    // By place where all places run at once: two layers of d 512, all rows of eight sequences of 300, 179.7 -> 177.8 us a step.  And where there
+    // are two at most and one tile is expected: no CTA has a pair then, and finding its number took each of them longer than the empty ones
+    // between do.  Four layers of d 4096, in turn / by place: 100 rows of five sequences of 215 positions 666 / 659 us, forward alone 21.7 / 20.5;
+    // 160 of eight x 215, 256 of three x 250, 400 of four x 256 and 800 of eight x 140 no difference.
+    const bool by_place = p.splits == 1 && (single < sms || (xtiles <= 2 && rows_seq <= tile_rows));
     p.places = p.splits > 1 ? clusters : by_place ? xtiles : 0;
-    cfg.gridDim = p.splits > 1 ? dim3(p.splits, heads, clusters * a.batch) : by_place ? dim3(single) : dim3((most > single ? most : single) + (p.split_last ? sms / 2 : 0));
+    cfg.gridDim = p.splits > 1 ? dim3(p.splits, heads, clusters * a.batch) : by_place ? dim3(heads * a.batch * xtiles) : dim3((most > single ? most : single) + (p.split_last ? sms / 2 : 0));
     cfg.blockDim = dim3(FWD_THREADS); cfg.dynamicSmemBytes = smem_fwd; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
