@@ -177,7 +177,10 @@ __device__ __noinline__ int4 forward_item(const int32_t* row_off, int batch, int
 }
 
 // kGroup: a tile has several query heads (one: the tile's divisions by their number fold away, 0.3 us of a CTA).
-template <bool kSplit, bool kGroup>
+// kOne: there are places for all tiles, so that a CTA has one tile at most, at its place.  (With the schedule for two in it as well a launch takes
+// 0.3 to 0.9 us longer: it is larger, and runs once.  Two layers of d 512, 194 rows of 570 positions 113.9 / 112.5 us a step, all of 300 in
+// eight sequences 178.7 / 176.7, four of d 4096, 40 rows of eight x 142 616 / 611.)
+template <bool kSplit, bool kGroup, bool kOne>
 __global__ void __launch_bounds__(FWD_THREADS, 1)
 attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const AttnTcParams p) {
@@ -194,14 +197,14 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   __shared__ int s_item[4];
   volatile int* item = s_item;
   if constexpr (kSplit) {
-    // The row tile is the slowest index, so that the live ones start first.  The grid may have room for half of the tiles only that there can
-    // be: with more rows than that every CTA takes two.  (Its other CTAs find nothing to do.)
+    // The row tile is the slowest index, so that the live ones start first.  Without kOne the grid has room for half of the tiles only that
+    // there can be: with more rows than that every CTA takes two.  (Its other CTAs find nothing to do.)
     const int b = (int)blockIdx.z % a.batch, r0 = a.row_off[b], nb = a.row_off[b + 1] - r0;
-    const int width = nb > p.places * tile_rows ? 2 * tile_rows : tile_rows, at = (int)blockIdx.z / a.batch * width;
+    const int width = !kOne && nb > p.places * tile_rows ? 2 * tile_rows : tile_rows, at = (int)blockIdx.z / a.batch * width;
     if (at >= nb) return;                                           // uniform in the cluster: nothing allocated yet
     if (threadIdx.x == 0) { item[0] = b; item[1] = blockIdx.y; item[2] = r0 + at; item[3] = min(width, nb - at); }
-  } else if (p.places > 0) {
-    // (by its place among `places` of each head where all places run at once: the numbering takes a CTA of several sequences 0.5 us)
+  } else if constexpr (kOne) {
+    // (by its place among `places` of each head: the numbering takes a CTA of several sequences 0.5 us)
     const int bg = div24(blockIdx.x, p.places), b = div24(bg, p.heads), r0 = a.row_off[b], at = ((int)blockIdx.x - bg * p.places) * tile_rows;
     const int nrows = min(tile_rows, a.row_off[b + 1] - r0 - at);
     if (nrows <= 0) return;
@@ -240,11 +243,11 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (!kSplit && item[3] <= 0) {
+  if (!kSplit && !kOne && item[3] <= 0) {
     if (warp == 1) tmem_dealloc(tmem_slot, 512);
     return;
   }
-  const int nq = item[3] > tile_rows ? 2 : 1;                          // live query tiles
+  const int nq = !kOne && item[3] > tile_rows ? 2 : 1;                          // live query tiles
   const uint32_t tm = tmem_slot;                                    // tile q: S/P at q*256, O at q*256 + 128
   volatile int* abortp = &abort_flag;
 
@@ -371,7 +374,7 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     if (q < nq) {
       const int quarter = warp & 3, lrow = q * AQ + quarter * 32 + lane;
       const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-      const bool dbuf = item[3] <= tile_rows;                            // one query tile: S/P alternate between the TMEM halves
+      const bool dbuf = kOne || item[3] <= tile_rows;                            // one query tile: S/P alternate between the TMEM halves
       const uint32_t to = tm + q * 256 + 128 + lane_base;
       const float sc = kLog2e * rsqrtf((float)ADH);
       float m_used = -INFINITY, l = 0.f;
@@ -553,10 +556,10 @@ attn_fwd_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     cluster_sync_all();
     if (warp >= 4 && !*abortp) {
       // this CTA's share of the tile's rows, a warp a row: the parts' sums relative to the largest of their maxima
-      const int first_live = min(item[3], tile_rows) * group, live = first_live + (item[3] > tile_rows ? (item[3] - tile_rows) * group : 0);
+      const int first_live = min(item[3], tile_rows) * group, live = first_live + (!kOne && item[3] > tile_rows ? (item[3] - tile_rows) * group : 0);
       const int ra = live * part / splits, rb = live * (part + 1) / splits;
       for (int n = ra + (warp - 4); n < rb; n += 8) {
-        const int q = n >= first_live ? 1 : 0, mine = n - q * first_live, r = q * AQ + mine, sel = kGroup ? div24(mine, group) : mine;
+        const int q = !kOne && n >= first_live ? 1 : 0, mine = n - q * first_live, r = q * AQ + mine, sel = kGroup ? div24(mine, group) : mine;
         const size_t at = (size_t)(item[2] + q * tile_rows + sel) * a.hq + item[1] * group + mine - sel * group;
         float pm[kMaxSplits], pl[kMaxSplits], m = -INFINITY, l = 0.f;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), x[kMaxSplits];
@@ -1024,7 +1027,8 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
   if (a.which != 2) {
     static PerDevice attr_set;
     if (attr_set.first()) {
-      for (auto* k : {attn_fwd_tc<false, false>, attn_fwd_tc<false, true>, attn_fwd_tc<true, false>, attn_fwd_tc<true, true>})
+      for (auto* k : {attn_fwd_tc<false, false, false>, attn_fwd_tc<false, true, false>, attn_fwd_tc<true, false, false>, attn_fwd_tc<true, true, false>,
+                      attn_fwd_tc<true, false, true>, attn_fwd_tc<true, true, true>, attn_fwd_tc<false, false, true>, attn_fwd_tc<false, true, true>})
         D2C_CUDA_OK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_fwd));
     }
     struct Maps { CUtensorMap q, k, v; } fresh, *m = &fresh;
@@ -1045,11 +1049,16 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     p.splits = splits_of(units);
     cudaLaunchConfig_t cfg = {};
     const int xtiles = ceil_div(a.max_rows_per_seq, tile_rows);
-    // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond; with shared keys, where no more than half of
-    // the tiles are expected, clusters for half of them, which take two each where that is not enough: 32 layers at 80 rows of 768 positions
-    // 3810 -> 3775 us against one for each, but two of d 512, all of 521 rows, 128 -> 134)
+    // (as many CTAs as there can be items: one a tile up to the SMs, one a pair of tiles beyond)
     const int most = heads * a.batch * ((xtiles + 1) / 2), single = heads * a.batch * xtiles < sms ? heads * a.batch * xtiles : sms;
-    const int clusters = 2 * ceil_div(rows_seq, tile_rows) > xtiles ? xtiles : (xtiles + 1) / 2;
+    // With shared keys there are places for all tiles where more than half of them are expected (two layers of d 512, all of 521 rows, 128 us,
+    // with places for half 134) or where the CTAs without rows are at most two waves behind the others; beyond, clusters for half of the tiles,
+    // which take two each where that is not enough.  Places for half / all, us: four layers, 28 heads over 4, 60 rows of 350 positions (252
+    // CTAs in all) 649 / 646, 500 (336) 645 / 634, 18 of 600 (420) 624 / 618, 32 heads 18 of 400 (384) 576 / 566; two of d 512, 100 rows of each
+    // of eight sequences of 300 (192) 144.0 / 140.5; but 32 heads 18 of 600 (480) 574 / 582, 28 heads 60 of 1024 (672) 644 / 649, 28 of 1390
+    // (924) 638 / 646; 32 layers at 80 of 768 (576) 3775 / 3810.
+    const bool one = 2 * ceil_div(rows_seq, tile_rows) > xtiles || (long long)p.splits * heads * a.batch * xtiles <= 3 * sms;
+    const int clusters = one ? xtiles : (xtiles + 1) / 2;
     if ((long long)clusters * a.batch > 65535) p.splits = 1;      // (tiles of a few rows, of many long sequences: the grid has no room for their places)
     const int pairs = ceil_div(ceil_div(rows_seq, tile_rows), 2) * heads * a.batch;      // (expected; where none are to be split, looking for them costs 0.4 us)
     p.split_last = units > sms && pairs > sms && pairs % sms > 0 && 2 * (pairs % sms) <= sms;
@@ -1067,7 +1076,10 @@ int launch_attention_tc(const AttnArgs& a, cudaStream_t st, int* status) {
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = p.splits; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = p.splits > 1 ? 2 : 1;
-    auto* kernel = p.splits > 1 ? (group > 1 ? attn_fwd_tc<true, true> : attn_fwd_tc<true, false>) : (group > 1 ? attn_fwd_tc<false, true> : attn_fwd_tc<false, false>);
+    auto* kernel = group > 1 ? attn_fwd_tc<false, true, false> : attn_fwd_tc<false, false, false>;
+    if (by_place) kernel = group > 1 ? attn_fwd_tc<false, true, true> : attn_fwd_tc<false, false, true>;
+    else if (p.splits > 1 && one) kernel = group > 1 ? attn_fwd_tc<true, true, true> : attn_fwd_tc<true, false, true>;
+    else if (p.splits > 1) kernel = group > 1 ? attn_fwd_tc<true, true, false> : attn_fwd_tc<true, false, false>;
     D2C_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, m->q, m->k, m->v, p));
     count_launch(1);
   }

@@ -182,3 +182,21 @@ def test_probabilities_of_few_rows_are_numbered_in_turn(runtime):
             forms.append({{name.split("AbarFormE")[1][0] for name in fake.fake_log().decode().split() if "AbarForm" in name}})
         assert forms == [{{"0"}}, {{"0"}}, {{"1"}}, {{"1"}}], (heads, seq, forms)
     """)
+
+
+def test_places_of_the_forward(runtime):
+    """Which form of the forward a step takes: with shared keys places for half of the tiles where those for all would be far more CTAs than
+    SMs, for all else; without, by place where one of two places is expected to be taken."""
+    from test_gpu_branches import PLACES
+    _run(runtime, f"""
+    def form(heads, kv, batch, seq, rows):
+        c = Ctx(replace(inputs.TOY_HD128, name="places", n_layers=1, n_q_heads=heads, n_kv_heads=kv), batch, seq)
+        for n in (batch * seq, rows, rows):
+            c.step(20, 0.0, n)
+        names = [n for n in fake.fake_log().decode().split() if "attn_fwd_tc" in n]
+        return names[0].split("attn_fwd_tc")[1][:13]
+    for want, heads, kv, seq in {PLACES}:
+        assert form(heads, kv, 1, seq, 20) == want, want
+    assert form(4, 2, 1, 570, 194) == "ILb1ELb0ELb1E"
+    assert form(32, 32, 5, 215, 100) == "ILb0ELb0ELb1E" and form(32, 32, 5, 700, 100) == "ILb0ELb0ELb0E"
+    """)
