@@ -356,25 +356,19 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
 #pragma unroll
           for (int i = 0; i < DH / 32; ++i) { qx[i] = ldcg16(qp + r0 * d_o + 32 * i); qy[i] = ldcg16(qp + r1 * d_o + 32 * i); }
           const float e0 = kLog2e * __ldcg(a.lse + (tile.x + r0) * hq + h), e1 = kLog2e * __ldcg(a.lse + (tile.x + r1) * hq + h);
-          // (as many keys at a time as there are registers for beside the weights of the product that follows)
-          constexpr int KJ = 256 / DH;
+          uint4 kf[4][DH / 32];
 #pragma unroll
-          for (int j0 = 0; j0 < 4; j0 += KJ) {
-            uint4 kf[KJ][DH / 32];
+          for (int j = 0; j < 4; ++j) {
+            const bf16* kp = kb + min(k0 + 8 * j + g8, L - 1) * kv_ld;
 #pragma unroll
-            for (int j = 0; j < KJ; ++j) {
-              const bf16* kp = kb + min(k0 + 8 * (j0 + j) + g8, L - 1) * kv_ld;
+            for (int i = 0; i < DH / 32; ++i) kf[j][i] = ldcg16(kp + 32 * i);
+          }
 #pragma unroll
-              for (int i = 0; i < DH / 32; ++i) kf[j][i] = ldcg16(kp + 32 * i);
-            }
+          for (int j = 0; j < 4; ++j) {
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int j = 0; j < KJ; ++j) {
-              float s[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-              for (int i = 0; i < DH / 32; ++i) mma_k32(s, qx[i], qy[i], kf[j][i]);
-              float* t4 = p[j0 + j];
-              t4[0] += ex2(s[0] * sc - e0); t4[1] += ex2(s[1] * sc - e0); t4[2] += ex2(s[2] * sc - e1); t4[3] += ex2(s[3] * sc - e1);
-            }
+            for (int i = 0; i < DH / 32; ++i) mma_k32(s, qx[i], qy[i], kf[j][i]);
+            p[j][0] += ex2(s[0] * sc - e0); p[j][1] += ex2(s[1] * sc - e0); p[j][2] += ex2(s[2] * sc - e1); p[j][3] += ex2(s[3] * sc - e1);
           }
         }
         float* to = s_p + (warp * 16 + g8) * 32 + 2 * q;
@@ -648,7 +642,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
           const bf16* qp = a.q + tile.x * d_o + h * DH + 8 * q;
           const int stride = 16 * ws;
           int k0 = 16 * split;
-          uint4 kf[2][DH / 32], v[DH / 64][4], qx[DH / 32], qy[DH / 32];
+          uint4 kf[2][DH / 32], v[4], qx[DH / 32], qy[DH / 32];
           auto load_k = [&](int at) {
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
@@ -660,9 +654,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
           auto load_v = [&](int at) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              const bf16* vp = vb + min(at + 2 * q + (i & 1) + 8 * (i >> 1), L - 1) * kv_ld;
-#pragma unroll
-              for (int x = 0; x < DH / 64; ++x) v[x][i] = ldcg16(vp + 64 * x);
+              v[i] = ldcg16(vb + min(at + 2 * q + (i & 1) + 8 * (i >> 1), L - 1) * kv_ld);
             }
           };
           {
@@ -671,11 +663,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
             for (int i = 0; i < DH / 32; ++i) { qx[i] = ldcg16(px + 32 * i); qy[i] = ldcg16(py + 32 * i); }
           }
           load_k(k0); load_v(k0);
-          float o[DH / 64][8][4], m0 = kNoKey, m1 = kNoKey, l0 = 0.f, l1 = 0.f;
+          float o[8][4], m0 = kNoKey, m1 = kNoKey, l0 = 0.f, l1 = 0.f;
 #pragma unroll
-          for (int x = 0; x < DH / 64; ++x)
-#pragma unroll
-            for (int i = 0; i < 8; ++i) o[x][i][0] = o[x][i][1] = o[x][i][2] = o[x][i][3] = 0.f;
+          for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
 #pragma unroll 1
           for (; k0 < L; k0 += stride) {
             float s[2][4];
@@ -706,17 +696,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
             l0 = l0 * c0 + (s[0][0] + s[0][1] + s[1][0] + s[1][1]);
             l1 = l1 * c1 + (s[0][2] + s[0][3] + s[1][2] + s[1][3]);
             const uint32_t pa[4] = {pack2(s[0][0], s[0][1]), pack2(s[0][2], s[0][3]), pack2(s[1][0], s[1][1]), pack2(s[1][2], s[1][3])};
-            // column g of product i is element 8 g + i of the head (of its second half): neighbouring elements of a lane's four rows
+            // column g of product i is element 8 g + i of the head: neighbouring elements of a lane's four rows
+            const uint32_t r[4][4] = {{v[0].x, v[0].y, v[0].z, v[0].w}, {v[1].x, v[1].y, v[1].z, v[1].w},
+                                      {v[2].x, v[2].y, v[2].z, v[2].w}, {v[3].x, v[3].y, v[3].z, v[3].w}};
 #pragma unroll
-            for (int x = 0; x < DH / 64; ++x) {
-              const uint32_t r[4][4] = {{v[x][0].x, v[x][0].y, v[x][0].z, v[x][0].w}, {v[x][1].x, v[x][1].y, v[x][1].z, v[x][1].w},
-                                        {v[x][2].x, v[x][2].y, v[x][2].z, v[x][2].w}, {v[x][3].x, v[x][3].y, v[x][3].z, v[x][3].w}};
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                o[x][i][0] *= c0; o[x][i][1] *= c0; o[x][i][2] *= c1; o[x][i][3] *= c1;
-                const uint32_t pick = (i & 1) ? 0x7632 : 0x5410;
-                mma16816(o[x][i], pa[0], pa[1], pa[2], pa[3], __byte_perm(r[0][i >> 1], r[1][i >> 1], pick), __byte_perm(r[2][i >> 1], r[3][i >> 1], pick));
-              }
+            for (int i = 0; i < 8; ++i) {
+              o[i][0] *= c0; o[i][1] *= c0; o[i][2] *= c1; o[i][3] *= c1;
+              const uint32_t pick = (i & 1) ? 0x7632 : 0x5410;
+              mma16816(o[i], pa[0], pa[1], pa[2], pa[3], __byte_perm(r[0][i >> 1], r[1][i >> 1], pick), __byte_perm(r[2][i >> 1], r[3][i >> 1], pick));
             }
             if (more) load_v(k0 + stride);
           }
@@ -725,12 +712,10 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1) small_step_k
           if (q == 0) { sml[warp * 16 + g8] = make_float2(m0, l0); sml[warp * 16 + g8 + 8] = make_float2(m1, l1); }
           float* to = so + (warp * 16 + g8) * SO + 16 * q;
 #pragma unroll
-          for (int x = 0; x < DH / 64; ++x)
+          for (int e = 0; e < 4; ++e)                          // c0, c1: row g; c2, c3: row g + 8
 #pragma unroll
-            for (int e = 0; e < 4; ++e)                        // c0, c1: row g; c2, c3: row g + 8
-#pragma unroll
-              for (int i = 0; i < 8; i += 4)
-                *reinterpret_cast<float4*>(to + 8 * (e >> 1) * SO + 64 * x + 8 * (e & 1) + i) = make_float4(o[x][i][e], o[x][i + 1][e], o[x][i + 2][e], o[x][i + 3][e]);
+            for (int i = 0; i < 8; i += 4)
+              *reinterpret_cast<float4*>(to + 8 * (e >> 1) * SO + 8 * (e & 1) + i) = make_float4(o[i][e], o[i + 1][e], o[i + 2][e], o[i + 3][e]);
         }
         __syncthreads();
         // a row's splits, side by side in a warp: the factor of each
