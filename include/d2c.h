@@ -31,13 +31,19 @@
  *     the caller's stream by events inside the call), so work enqueued on the
  *     caller's stream after the call still sees the whole step; D2C_FLAG_SERIAL
  *     keeps every kernel on the caller's stream.  A small model's step is one
- *     cooperative launch on it, which takes most SMs at once.  Any step can be captured
+ *     cooperative launch on it, which takes most SMs at once, so that no other step runs
+ *     beside it: a step of each of two contexts on two streams takes 72 us of the GPU, in
+ *     separate kernels 58 (one layer of d 256, 95 rows; one context by itself 37 and 49), of
+ *     three layers 166 and 118 (87 and 108).  Programs that keep several small models busy
+ *     at once ask for separate kernels with D2C_FLAG_FOLDED_NORMS.  Any step can be captured
  *     into a CUDA graph from the caller's stream and replayed (the choice between
  *     kernel variants that follows an earlier step's row count is then frozen).
  *     One context per stream; a context is not re-entrant.
  *   - What a step computes does not depend on the steps before it, but its last bits
  *     do: the row count of the previous step (none in a capture) decides how sums are
- *     split and whether the RMSNorms are folded into the projections.  Behind steps of
+ *     split, whether the RMSNorms are folded into the projections and, unless the call asks
+ *     for more rows of stage 1 or more of the mass than that step did, whether a small
+ *     model's step is one launch.  Behind steps of
  *     one size the same inputs and state give the same bits; behind others the results
  *     differ within the roundings to bf16 (hidden states by up to 2e-3 of a row's norm
  *     in one or two layers).
@@ -87,7 +93,8 @@ typedef struct {
 #define D2C_FLAG_FOLDED_NORMS 16        /* fold the layers' RMSNorms into the GEMM epilogues around them (x * gain and the row's sums of
                                            squares written by the residual epilogue, the row scale applied by the next projection)
                                            instead of running them as kernels of their own; a step that expects few rows (at most 128, going
-                                           by the previous step) does so without the flag, which moves its results by roundings       */
+                                           by the previous step) does so without the flag, which moves its results by roundings.  With any
+                                           flag but SERIAL a small model's step is never one launch            */
 
 /* Weights.  The arrays of per-layer pointers are HOST arrays of n_layers DEVICE
  * pointers; they are copied at create, the device memory is borrowed for the
@@ -208,6 +215,7 @@ int d2c_sync_status(d2c_ctx* ctx);
 
 /* Per-phase timing of d2c_step.  While enabled, d2c_step records one CUDA event at every phase
  * boundary on the context's stream (events are host objects; no device memory is allocated).
+ * One launch for a whole step has no such boundaries: small models then run the separate kernels.
  * d2c_profile_read synchronises the stream and returns, accumulated since the last reset, the
  * milliseconds spent in each phase (phase_ms[D2C_N_PHASES]) and the number of kernels the library
  * launched in it (phase_launches[D2C_N_PHASES]); either may be NULL.  d2c_phase_name(i) names

@@ -1,13 +1,14 @@
 // Selected-query bidirectional attention on the 5th-generation tensor cores (head_dim 128).
 //
 //   attn_fwd_tc    O = softmax(Q K^T / sqrt(Dh)) V and the log-sum-exp per (row, head).  One CTA per
-//                  (256 selected rows, head, sequence); keys stream in tiles of 128 through TMA.
+//                  one or two tiles of up to 128 (selected row, query head) pairs of a K/V head and a
+//                  sequence; keys stream in tiles of 128 through TMA.
 //                  S = Q K^T is a tcgen05.mma into TMEM; softmax warps (one row per thread) read it
 //                  with tcgen05.ld, write the bf16 probabilities back over the same TMEM columns and the
 //                  PV product takes them from there as its A operand (V is the MN-major B operand straight
 //                  from the TMA tile) and accumulates O in TMEM.
 //   attn_abar_tc   Abar[r][j] = 1/Hq sum_h exp(s_h[r][j] - lse_h[r]) (Section 4.2): one pair of CTAs per
-//                  (256 keys x up to 256 rows) loops over the heads, S^T by tcgen05.mma, the sum over heads in
+//                  (256 keys x up to 256 rows) loops over heads, S^T by tcgen05.mma, the sum over heads in
 //                  registers in a fixed order (deterministic).
 //
 // Warp roles in both: warp 0 TMA producer, warp 1 MMA issuer + TMEM owner, warps 4..11 softmax/epilogue.
@@ -63,8 +64,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 struct AttnTcParams { AttnArgs a; int* status; int sm_count; int splits, head_groups, row_tile, pairs; int group, heads, kv_share, rows, split_last, places; };      // group: query heads of a tile, of the same K/V head; heads: such groups; kv_share: those of a K/V head; rows: selected rows of a query tile; places: tiles of a sequence's head that the grid has places for (0: numbered in turn)
 
 // ------------------------------------------------------------------------------------------------
-// Forward kernel.  One CTA owns up to 256 selected rows of one (sequence, head): two query tiles of
-// 128 rows that share every K/V tile brought in by TMA.  Each query tile has its own softmax warp
+// Forward kernel.  One CTA owns up to two query tiles of one (sequence, K/V head), which share every K/V
+// tile brought in by TMA.  A tile's 128 rows are `rows` selected rows x `group` query heads of that K/V head, the
+// head the faster (18 x 7, two rows unused), or 128 selected rows of one head.  Each query tile has its own softmax warp
 // group (4 warps, one row per thread) and its own TMEM columns: 128 for the scores S (overwritten in
 // place by the bf16 probabilities P) and 128 for the output accumulator O, which stays in TMEM across
 // the key tiles.  The running maximum is only raised when it grows by more than 2^8 (P stays exactly
@@ -943,7 +945,7 @@ static int expected_rows_per_seq(const AttnArgs& a) {
 
 struct AbarCut { int hgs, row_tile, ctas, waves; };
 static AbarCut abar_cut(const AttnArgs& a, float* us = nullptr) {
-  // How the work is cut: row tiles of 64, 128 or 256 rows, heads shared by 1, 2 or 4 pairs (whole kv groups each); the
+  // How the work is cut: row tiles of 64, 128 or 256 rows (or any multiple of 16, see below), heads shared by 1, 2 or 4 pairs (whole kv groups each); the
   // cheapest by this estimate of waves x time of a CTA (us, measured: a head of a 256-row tile takes 1.8, of a narrow one
   // the loads' 0.5; 6 for set-up, first loads and output; 2 for the meeting).  The row count is an expectation (worst case
   // if there is none): it decides how the work is cut, not what is covered.  Beside other kernels the fewest SMs are best.

@@ -160,7 +160,7 @@ struct d2c_ctx {
   int32_t* hint_dev[2] = {nullptr, nullptr};
   cudaEvent_t ev_hint[2] = {nullptr, nullptr};
   long long hint_step[2] = {-1, -1};     // step number whose count the word holds
-  bool hint_tagged[2] = {false, false};  // it was a step in one launch: it writes its number behind the count, in one store
+  bool hint_tagged[2] = {false, false};  // it was a step in one launch: it writes its number and the count as one 64-bit word
   long long step_no = 0;
   int asked_k = 0; float asked_p = 0.f;  // rows of stage 1 at most, and mass of stage 2, that the step before asked for
   bool few_rows = false;                 // this step's regime: at most 128 rows expected
@@ -530,7 +530,9 @@ static CopyOut index_outputs(const d2c_ctx* ctx, const d2c_step_out* out, int ro
 // the rows are a part of the room only and so mostly known ones, without work for the LM head.  (us, one launch / separate kernels, one layer
 // of d 256: 61 rows of 256 positions 40 / 60, 216 of 600 56 / 71, 224 of 16 x 300 60 / 75, all of 112 rows 41 / 86, all of 224 in four
 // sequences, three tiles, 56 / 55, with 4096 columns of the LM head 71 / 58; two of d 384: 109 of 256 73 / 90, all of 112 70 / 181, 125 rows, two
-// tiles, 93 / 88; three of d 512: 106 of 600 128 / 151, 125 rows 135 / 124.)
+// tiles, 93 / 88; three of d 512: 106 of 600 128 / 151, 125 rows 135 / 124.  One layer of d 256 with 1500 columns, 110 rows, 51 / 66, with 2048
+// 52 / 67, all 221 masked in part 61 / 70; of four and eight layers, d 256 to 512, 59 to 328 rows of 256 to 3000 positions, one to four
+// sequences, the one launch is ahead by 4 % (four of d 512, 59 rows, 153 / 160) to 35 % (eight of d 256, 110 rows, 250 / 337).)
 static bool few_for_one_launch(const d2c_ctx* ctx, int batch, int room, int rows) {
   const d2c_config& c = ctx->cfg;
   const int most = c.d_model > 256 || (long long)c.vocab * c.d_model > 1 << 18 ? 1 : 2 * rows <= room ? 3 : 2;
